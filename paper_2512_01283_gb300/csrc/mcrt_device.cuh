@@ -37,15 +37,39 @@ __device__ __forceinline__ void t_sincospi(double x, double* s, double* c) { sin
 __device__ __forceinline__ void t_sincos(float x, float* s, float* c) { sincosf(x, s, c); }
 __device__ __forceinline__ void t_sincos(double x, double* s, double* c) { sincos(x, s, c); }
 
+// Sums of two products a b + c d in a stated rounding: one product is fused into the
+// addition of the other, which is rounded.  Left to the compiler (kFree), the product that
+// is fused depends on the code around the expression, so that the same formula rounds
+// differently from one version of a kernel to the next and FP32 trajectories part.  The
+// choices below, and those of the call sites, are the ones that keep every packet's
+// trajectory, tally and image what they have been.
+enum Fuse { kFirst, kSecond, kFree };
+__device__ __forceinline__ float t_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double t_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float t_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double t_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float t_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double t_add(double a, double b) { return __dadd_rn(a, b); }
+// a b + c d and a b - c d
+template <Fuse F = kFirst, typename T> __device__ __forceinline__ T mad2(T a, T b, T c, T d) {
+    if constexpr (F == kFree) return a * b + c * d;
+    return F == kSecond ? t_fma(c, d, t_mul(a, b)) : t_fma(a, b, t_mul(c, d));
+}
+template <Fuse F = kFirst, typename T> __device__ __forceinline__ T msb2(T a, T b, T c, T d) {
+    if constexpr (F == kFree) return a * b - c * d;
+    return mad2<F>(a, b, -c, d);
+}
+
 template <typename T> struct V3 {
     T x, y, z;
 };
 template <typename T> __device__ __forceinline__ V3<T> v3(T x, T y, T z) { return V3<T>{x, y, z}; }
-template <typename T> __device__ __forceinline__ T dot(const V3<T>& a, const V3<T>& b) {
-    return a.x * b.x + a.y * b.y + a.z * b.z;
+template <Fuse F = kFirst, typename T> __device__ __forceinline__ T dot(const V3<T>& a, const V3<T>& b) {
+    if constexpr (F == kFree) return a.x * b.x + a.y * b.y + a.z * b.z;
+    return t_fma(a.z, b.z, mad2<F>(a.x, b.x, a.y, b.y));
 }
-template <typename T> __device__ __forceinline__ V3<T> cross(const V3<T>& a, const V3<T>& b) {
-    return V3<T>{a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+template <Fuse F = kFirst, typename T> __device__ __forceinline__ V3<T> cross(const V3<T>& a, const V3<T>& b) {
+    return V3<T>{msb2<F>(a.y, b.z, a.z, b.y), msb2<F>(a.z, b.x, a.x, b.z), msb2<F>(a.x, b.y, a.y, b.x)};
 }
 template <typename T> __device__ __forceinline__ V3<T> axpy(T s, const V3<T>& a, const V3<T>& b) {
     return V3<T>{s * a.x + b.x, s * a.y + b.y, s * a.z + b.z};
@@ -111,18 +135,18 @@ __device__ __forceinline__ Draw4<T> draw4(long long pid, uint32_t event, uint32_
 //   to_lab:   q (0,v) q^*  = v + 2 s (w x v) + 2 w x (w x v)
 //   to_grain: q^* (0,v) q  = v - 2 s (w x v) + 2 w x (w x v)
 // ---------------------------------------------------------------------------------
-template <typename T> __device__ __forceinline__ V3<T> quat_to_lab(const float4& q, const V3<T>& v) {
+template <Fuse F = kFirst, typename T> __device__ __forceinline__ V3<T> quat_to_lab(const float4& q, const V3<T>& v) {
     const V3<T> w{T(q.y), T(q.z), T(q.w)};
     const T s = T(q.x);
-    const V3<T> t = cross(w, v);
-    const V3<T> tt = cross(w, t);
+    const V3<T> t = cross<F>(w, v);
+    const V3<T> tt = cross<F>(w, t);
     return V3<T>{v.x + T(2) * (s * t.x + tt.x), v.y + T(2) * (s * t.y + tt.y), v.z + T(2) * (s * t.z + tt.z)};
 }
-template <typename T> __device__ __forceinline__ V3<T> quat_to_grain(const float4& q, const V3<T>& v) {
+template <Fuse F = kFirst, typename T> __device__ __forceinline__ V3<T> quat_to_grain(const float4& q, const V3<T>& v) {
     const V3<T> w{T(q.y), T(q.z), T(q.w)};
     const T s = T(q.x);
-    const V3<T> t = cross(w, v);
-    const V3<T> tt = cross(w, t);
+    const V3<T> t = cross<F>(w, v);
+    const V3<T> tt = cross<F>(w, t);
     return V3<T>{v.x + T(2) * (tt.x - s * t.x), v.y + T(2) * (tt.y - s * t.y), v.z + T(2) * (tt.z - s * t.z)};
 }
 
@@ -130,15 +154,16 @@ template <typename T> __device__ __forceinline__ V3<T> quat_to_grain(const float
 // Stokes basis of n without trigonometry: phi-hat = (-n_y, n_x, 0) / rho,
 // theta-hat = phi-hat x n; at the poles phi-hat = (0, 1, 0).
 // ---------------------------------------------------------------------------------
-template <typename T> __device__ __forceinline__ void stokes_basis(const V3<T>& n, V3<T>& th, V3<T>& ph) {
-    const T r2 = n.x * n.x + n.y * n.y;
+template <Fuse F = kFirst, typename T>
+__device__ __forceinline__ void stokes_basis(const V3<T>& n, V3<T>& th, V3<T>& ph) {
+    const T r2 = mad2<F>(n.x, n.x, n.y, n.y);
     if (r2 > T(0)) {
         const T r = t_rsqrt(r2);
         ph = V3<T>{-n.y * r, n.x * r, T(0)};
     } else {
         ph = V3<T>{T(0), T(1), T(0)};
     }
-    th = cross(ph, n);
+    th = cross<F == kFree ? kFree : kFirst>(ph, n);
 }
 
 __device__ __forceinline__ float t_rcp(float x) { return __fdividef(1.0f, x); }
@@ -149,8 +174,8 @@ __device__ __forceinline__ double t_div(double a, double b) { return a / b; }
 
 // (cos 2psi, sin 2psi) from any (A, B) proportional to (cos psi, sin psi); (1, 0)
 // for A = B = 0.  Tiny inputs are rescaled first so that 1/r cannot overflow.
-template <typename T> __device__ __forceinline__ void double_angle(T A, T B, T& c2, T& s2) {
-    T r = A * A + B * B;
+template <Fuse F = kFirst, typename T> __device__ __forceinline__ void double_angle(T A, T B, T& c2, T& s2) {
+    T r = mad2<F>(A, A, B, B);
     if (!(r >= T(1e-30))) {
         const T m = fmax(fabs(A), fabs(B));
         if (!(m > T(0))) {
@@ -160,17 +185,23 @@ template <typename T> __device__ __forceinline__ void double_angle(T A, T B, T& 
         }
         A = A / m;
         B = B / m;
-        r = A * A + B * B;
+        r = mad2<F>(A, A, B, B);
     }
     const T inv = t_rcp(r);
-    c2 = (A * A - B * B) * inv;
+    c2 = msb2<F>(A, A, B, B) * inv;
     s2 = T(2) * A * B * inv;
 }
 
-// eq. (stokes-rotation): (Q', U') = [[c2, s2], [-s2, c2]] (Q, U)
-template <typename T> __device__ __forceinline__ void rotate_qu(T& Q, T& U, T c2, T s2) {
-    const T q = c2 * Q + s2 * U;
-    const T u = -s2 * Q + c2 * U;
+// eq. (stokes-rotation): (Q', U') = [[c2, s2], [-s2, c2]] (Q, U), and back
+template <Fuse F = kFirst, typename T> __device__ __forceinline__ void rotate_qu(T& Q, T& U, T c2, T s2) {
+    const T q = mad2<F>(c2, Q, s2, U);
+    const T u = msb2(c2, U, s2, Q);
+    Q = q;
+    U = u;
+}
+template <typename T> __device__ __forceinline__ void rotate_back(T& Q, T& U, T c2, T s2) {
+    const T q = msb2(c2, Q, s2, U);
+    const T u = mad2(s2, Q, c2, U);
     Q = q;
     U = u;
 }
@@ -181,15 +212,15 @@ template <typename T> struct GrainFrame {
     T c2, s2, cos_tp;
 };
 
-template <typename T>
+template <Fuse F = kFirst, typename T>
 __device__ __forceinline__ GrainFrame<T> grain_frame(const float4& q, const V3<T>& n, const V3<T>& ph_lab) {
     const V3<T> nGF = quat_to_grain(q, n);
     const V3<T> phGF = quat_to_grain(q, ph_lab);
     // phi' of n_GF up to a positive factor; (0, 1, 0) along the grain axis
     V3<T> php{-nGF.y, nGF.x, T(0)};
     if (php.x == T(0) && php.y == T(0)) php.y = T(1);
-    const T cos_eta = dot(phGF, php);
-    const T sin_eta = dot(cross(phGF, php), nGF);
+    const T cos_eta = mad2<kSecond>(phGF.x, php.x, phGF.y, php.y);
+    const T sin_eta = dot<F>(cross<F>(phGF, php), nGF);
     GrainFrame<T> f;
     double_angle(cos_eta, sin_eta, f.c2, f.s2);
     f.cos_tp = nGF.z;
@@ -232,54 +263,98 @@ template <typename T> __device__ __forceinline__ void e1_complex(T x, T y, T& re
     (void)cy;
 }
 
-// Y = e^{-M dtau} X; with want_W also W = wscale * int_0^1 e^{-M dtau s} ds X
-// (wscale = dtau gives the optical-depth integral, wscale = ell the path-length one,
-// which needs no division by kappa_ext).  For |a2 dtau| <= 10 the I-Q block uses the
-// cosh/sinh form of App. A (no cancellation in Q); beyond, the eigen-decay form, whose
-// factors underflow to zero instead of overflowing.
-template <typename T>
-__device__ __forceinline__ void transfer(const T X[4], T a, T a2, T a3, T dtau, T Y[4], T W[4], bool want_W,
-                                         T wscale) {
-    const T xa = a * dtau, xb = a2 * dtau, ya = a3 * dtau;
-    const T xp = xa + xb, xm = xa - xb;
-    const T ea = t_exp(-xa);
-    if (fabs(xb) <= T(10)) {
+// The coefficients of Y = e^{-M dtau} X.  For |a2 dtau| <= 10 the I-Q block uses the
+// cosh/sinh form of App. A (no cancellation in Q); beyond (thick), the eigen-decay form,
+// whose factors (ch, sh = e^{-xp}, e^{-xm}) underflow to zero instead of overflowing.
+template <typename T> struct Decay {
+    T ea, ch, sh, c3, s3;
+    bool thick;
+};
+
+template <typename T> __device__ __forceinline__ Decay<T> decay_of(T xa, T xb, T ya, T xp, T xm) {
+    Decay<T> d;
+    d.ea = t_exp(-xa);
+    d.thick = !(fabs(xb) <= T(10));
+    if (!d.thick) {
         // e^{-xb} - 1 = -m / (1 + m) with m = e^{xb} - 1: no cancellation, one expm1
         const T e1p = t_expm1(xb), e1m = -e1p * t_rcp(T(1) + e1p);
-        const T sh = T(0.5) * (e1p - e1m), ch = T(1) + T(0.5) * (e1p + e1m);
-        Y[0] = ea * (ch * X[0] - sh * X[1]);
-        Y[1] = ea * (ch * X[1] - sh * X[0]);
+        d.sh = T(0.5) * (e1p - e1m);
+        d.ch = T(1) + T(0.5) * (e1p + e1m);
+    } else {
+        d.ch = t_exp(-xp);
+        d.sh = t_exp(-xm);
+    }
+    d.s3 = T(0);
+    d.c3 = T(1);
+    if (ya != T(0)) t_sincos(ya, &d.s3, &d.c3);
+    return d;
+}
+
+// Y = e^{-M dtau} X
+template <typename T> __device__ __forceinline__ void apply_decay(const Decay<T>& d, const T X[4], T Y[4]) {
+    if (!d.thick) {
+        Y[0] = t_mul(d.ea, msb2(d.ch, X[0], d.sh, X[1]));
+        Y[1] = t_mul(d.ea, msb2(d.ch, X[1], d.sh, X[0]));
     } else {
         const T sp = X[0] + X[1], sm = X[0] - X[1];
-        const T ep = t_exp(-xp), em = t_exp(-xm);
-        Y[0] = T(0.5) * (ep * sp + em * sm);
-        Y[1] = T(0.5) * (ep * sp - em * sm);
+        Y[0] = T(0.5) * mad2(d.ch, sp, d.sh, sm);
+        Y[1] = T(0.5) * msb2(d.ch, sp, d.sh, sm);
     }
-    T s3 = T(0), c3 = T(1);
-    if (ya != T(0)) t_sincos(ya, &s3, &c3);
-    Y[2] = ea * (c3 * X[2] - s3 * X[3]);
-    Y[3] = ea * (s3 * X[2] + c3 * X[3]);
-    if (want_W) {
-        const T sp = X[0] + X[1], sm = X[0] - X[1];
-        const T Ep = wscale * e1(xp), Em = wscale * e1(xm);
-        W[0] = T(0.5) * (Ep * sp + Em * sm);
-        W[1] = T(0.5) * (Ep * sp - Em * sm);
-        T re, im;
-        e1_complex(xa, ya, re, im);
-        re *= wscale;
-        im *= wscale;
-        W[2] = re * X[2] - im * X[3];
-        W[3] = re * X[3] + im * X[2];
-    }
+    Y[2] = t_mul(d.ea, msb2(d.c3, X[2], d.s3, X[3]));
+    Y[3] = t_mul(d.ea, mad2<kSecond>(d.s3, X[2], d.c3, X[3]));
+}
+
+// W = wscale * int_0^1 e^{-M dtau s} ds X (wscale = dtau gives the optical-depth integral,
+// wscale = ell the path-length one, which needs no division by kappa_ext)
+template <typename T>
+__device__ __forceinline__ void path_integral(T xa, T ya, T xp, T xm, const T X[4], T W[4], T wscale) {
+    const T sp = X[0] + X[1], sm = X[0] - X[1];
+    const T Ep = t_mul(wscale, e1(xp)), Em = t_mul(wscale, e1(xm));
+    W[0] = T(0.5) * mad2(Ep, sp, Em, sm);
+    W[1] = T(0.5) * msb2(Ep, sp, Em, sm);
+    T re, im;
+    e1_complex(xa, ya, re, im);
+    re = t_mul(re, wscale);
+    im = t_mul(im, wscale);
+    W[2] = msb2(re, X[2], im, X[3]);
+    W[3] = mad2<kSecond>(re, X[3], im, X[2]);
+}
+
+// A segment's Y = e^{-M dtau} X and, with want_W, its path integral W.
+template <bool fused_xm = false, typename T>
+__device__ __forceinline__ void transfer(const T X[4], T a, T a2, T a3, T dtau, T Y[4], T W[4], bool want_W,
+                                         T wscale) {
+    const T xa = t_mul(a, dtau), xb = t_mul(a2, dtau), ya = t_mul(a3, dtau);
+    const T xp = t_fma(a2, dtau, xa), xm = fused_xm ? t_fma(a, dtau, -xb) : t_add(xa, -xb);
+    apply_decay(decay_of(xa, xb, ya, xp, xm), X, Y);
+    if (want_W) path_integral(xa, ya, xp, xm, X, W, wscale);
 }
 
 // Full App. A cell step with source S (per unit dtau) and the extinction matrix K:
-// X <- e^{-K dtau} X + (int_0^dtau e^{-K t} dt) S
-template <typename T> __device__ __forceinline__ void cell_step(T X[4], T a1, T a2, T a3, const T S[4], T dtau) {
-    T Y[4], W[4], Z[4];
-    transfer(X, a1, a2, a3, dtau, Y, W, false, dtau);
-    transfer(S, a1, a2, a3, dtau, Z, W, true, dtau);
-    for (int e = 0; e < 4; ++e) X[e] = Y[e] + W[e];
+// X <- e^{-K dtau} X + (int_0^dtau e^{-K t} dt) S.  Its coefficients do not depend on X.
+template <typename T> struct CellStep {
+    Decay<T> d;
+    T W[4];
+};
+template <typename T> __device__ __forceinline__ CellStep<T> cell_coeffs(T a1, T a2, T a3, const T S[4], T dtau) {
+    const T xa = t_mul(a1, dtau), xb = t_mul(a2, dtau), ya = t_mul(a3, dtau);
+    const T xm = t_add(xa, -xb);
+    CellStep<T> c;
+    c.d = decay_of(xa, xb, ya, t_fma(a2, dtau, xa), xm);
+    path_integral(xa, ya, t_add(xa, xb), xm, S, c.W, dtau);
+    return c;
+}
+template <typename T> __device__ __forceinline__ void cell_step(const CellStep<T>& c, T X[4]) {
+    T Y[4];
+    apply_decay(c.d, X, Y);
+    Y[0] = t_add(Y[0], c.W[0]);
+    Y[1] = t_add(Y[1], c.W[1]);
+    const T u = t_fma(c.d.ea, msb2(c.d.c3, X[2], c.d.s3, X[3]), c.W[2]);
+    const T v = t_fma(c.d.ea, mad2(c.d.s3, X[2], c.d.c3, X[3]), c.W[3]);
+    X[0] = Y[0];
+    X[1] = Y[1];
+    X[2] = u;
+    X[3] = v;
 }
 
 // ---------------------------------------------------------------------------------
@@ -305,20 +380,20 @@ template <typename T> struct PlaneRot {
 
 // With e = n x n2 the rotation inputs are projections: e.phi(n) = n2.theta(n),
 // -e.theta(n) = n2.phi(n), e.phi(n2) = -n.theta(n2), e.theta(n2) = n.phi(n2).
-template <typename T>
+template <Fuse F = kFirst, Fuse FA1 = F, Fuse FA2 = F, typename T>
 __device__ __forceinline__ PlaneRot<T> plane_rotation(const V3<T>& n, const V3<T>& th, const V3<T>& ph,
                                                       const V3<T>& n2, const V3<T>& th2, const V3<T>& ph2) {
-    T A1 = dot(n2, th), B1 = dot(n2, ph);
-    T A2 = -dot(n, th2), B2 = dot(n, ph2);
-    if (A1 * A1 + B1 * B1 < T(1e-12)) {  // sin(Theta) < 1e-6: plane undefined, e_perp = phi(n)
+    T A1 = dot<FA1>(n2, th), B1 = dot<F>(n2, ph);
+    T A2 = -dot<FA2>(n, th2), B2 = dot<F>(n, ph2);
+    if (mad2<F>(A1, A1, B1, B1) < T(1e-12)) {  // sin(Theta) < 1e-6: plane undefined, e_perp = phi(n)
         A1 = T(1);
         B1 = T(0);
-        A2 = dot(ph, ph2);
-        B2 = dot(ph, th2);
+        A2 = dot<F>(ph, ph2);
+        B2 = dot<F>(ph, th2);
     }
     PlaneRot<T> r;
-    double_angle(A1, B1, r.c1, r.s1);
-    double_angle(A2, B2, r.c2, r.s2);
+    double_angle<F>(A1, B1, r.c1, r.s1);
+    double_angle<F>(A2, B2, r.c2, r.s2);
     return r;
 }
 
@@ -326,22 +401,23 @@ __device__ __forceinline__ PlaneRot<T> plane_rotation(const V3<T>& n, const V3<T
 template <typename T>
 __device__ __forceinline__ T plane_Q(const V3<T>& th, const V3<T>& ph, const V3<T>& n2, const T X[4]) {
     const T A1 = dot(n2, th), B1 = dot(n2, ph);
-    if (A1 * A1 + B1 * B1 < T(1e-12)) return X[1];
+    if (mad2(A1, A1, B1, B1) < T(1e-12)) return X[1];
     T c1, s1;
     double_angle(A1, B1, c1, s1);
-    return c1 * X[1] + s1 * X[2];
+    return mad2(c1, X[1], s1, X[2]);
 }
 
-template <typename T> __device__ __forceinline__ void apply_plane(const PlaneRot<T>& r, const T P[6], const T X[4], T Y[4]) {
-    const T Qs = r.c1 * X[1] + r.s1 * X[2];
-    const T Us = -r.s1 * X[1] + r.c1 * X[2];
-    const T I2 = P[0] * X[0] + P[1] * Qs;
-    const T Q2 = P[1] * X[0] + P[2] * Qs;
-    const T U2 = P[3] * Us + P[4] * X[3];
-    const T V2 = -P[4] * Us + P[5] * X[3];
+template <Fuse F = kFirst, Fuse FI = F, typename T>
+__device__ __forceinline__ void apply_plane(const PlaneRot<T>& r, const T P[6], const T X[4], T Y[4]) {
+    const T Qs = mad2<F>(r.c1, X[1], r.s1, X[2]);
+    const T Us = F == kFree ? -r.s1 * X[1] + r.c1 * X[2] : msb2(r.c1, X[2], r.s1, X[1]);
+    const T I2 = mad2<FI>(P[0], X[0], P[1], Qs);
+    const T Q2 = mad2<F>(P[1], X[0], P[2], Qs);
+    const T U2 = mad2<F == kFree ? kFree : kSecond>(P[3], Us, P[4], X[3]);
+    const T V2 = F == kFree ? -P[4] * Us + P[5] * X[3] : msb2(P[5], X[3], P[4], Us);
     Y[0] = I2;
-    Y[1] = r.c2 * Q2 + r.s2 * U2;
-    Y[2] = -r.s2 * Q2 + r.c2 * U2;
+    Y[1] = mad2<F>(r.c2, Q2, r.s2, U2);
+    Y[2] = F == kFree ? -r.s2 * Q2 + r.c2 * U2 : msb2(r.c2, U2, r.s2, Q2);
     Y[3] = V2;
 }
 
@@ -370,30 +446,30 @@ __device__ __forceinline__ void dipole_K(T ca0, T ca1, T cs0, T cs1, T fa, T fs,
 // alpha'_0 (1 + (rho - 1) ax ax^T) E and the far field along n2 its transverse part, so
 // the Jones matrix is J_jk = f2_j . f_k + (rho - 1) (f2_j . ax)(ax . f_k); the coherency
 // matrix C = 1/2 [[I+Q, U+iV], [U-iV, I-Q]] goes to J C J^H, scaled by zn.
-template <typename T>
+template <Fuse F = kFirst, typename T>
 __device__ __forceinline__ void dipole_apply(T rho_re, T rho_im, T zn, const V3<T>& ax, const V3<T>& th,
                                              const V3<T>& ph, const V3<T>& th2, const V3<T>& ph2, const T X[4],
                                              T Y[4]) {
     const T rr = rho_re - T(1);
     const T g0 = dot(th2, ax), g1 = dot(ph2, ax), b0 = dot(ax, th), b1 = dot(ax, ph);
     // J = (Jr + i Ji)
-    const T Jr00 = dot(th2, th) + rr * g0 * b0, Ji00 = rho_im * g0 * b0;
-    const T Jr01 = dot(th2, ph) + rr * g0 * b1, Ji01 = rho_im * g0 * b1;
+    const T Jr00 = dot<F>(th2, th) + rr * g0 * b0, Ji00 = rho_im * g0 * b0;
+    const T Jr01 = dot<F>(th2, ph) + rr * g0 * b1, Ji01 = rho_im * g0 * b1;
     const T Jr10 = dot(ph2, th) + rr * g1 * b0, Ji10 = rho_im * g1 * b0;
     const T Jr11 = dot(ph2, ph) + rr * g1 * b1, Ji11 = rho_im * g1 * b1;
     // C (Hermitian): c00, c11 real, c01 = cr + i ci, c10 = conj(c01)
     const T c00 = T(0.5) * (X[0] + X[1]), c11 = T(0.5) * (X[0] - X[1]);
     const T cr = T(0.5) * X[2], ci = T(0.5) * X[3];
     // M = J C
-    const T Mr00 = Jr00 * c00 + Jr01 * cr + Ji01 * ci, Mi00 = Ji00 * c00 + Ji01 * cr - Jr01 * ci;
-    const T Mr01 = Jr00 * cr - Ji00 * ci + Jr01 * c11, Mi01 = Jr00 * ci + Ji00 * cr + Ji01 * c11;
-    const T Mr10 = Jr10 * c00 + Jr11 * cr + Ji11 * ci, Mi10 = Ji10 * c00 + Ji11 * cr - Jr11 * ci;
-    const T Mr11 = Jr10 * cr - Ji10 * ci + Jr11 * c11, Mi11 = Jr10 * ci + Ji10 * cr + Ji11 * c11;
+    const T Mr00 = t_fma(Ji01, ci, mad2(Jr00, c00, Jr01, cr)), Mi00 = t_fma(-Jr01, ci, mad2(Ji00, c00, Ji01, cr));
+    const T Mr01 = t_fma(Jr01, c11, msb2(Jr00, cr, Ji00, ci)), Mi01 = t_fma(Ji01, c11, mad2<kSecond>(Jr00, ci, Ji00, cr));
+    const T Mr10 = t_fma(Ji11, ci, mad2(Jr10, c00, Jr11, cr)), Mi10 = t_fma(-Jr11, ci, mad2(Ji10, c00, Ji11, cr));
+    const T Mr11 = t_fma(Jr11, c11, msb2(Jr10, cr, Ji10, ci)), Mi11 = t_fma(Ji11, c11, mad2<kSecond>(Jr10, ci, Ji10, cr));
     // D = M J^H: D_jk = sum_l M_jl conj(J_kl)
-    const T D00 = Mr00 * Jr00 + Mi00 * Ji00 + Mr01 * Jr01 + Mi01 * Ji01;
-    const T D11 = Mr10 * Jr10 + Mi10 * Ji10 + Mr11 * Jr11 + Mi11 * Ji11;
-    const T Dr01 = Mr00 * Jr10 + Mi00 * Ji10 + Mr01 * Jr11 + Mi01 * Ji11;
-    const T Di01 = Mi00 * Jr10 - Mr00 * Ji10 + Mi01 * Jr11 - Mr01 * Ji11;
+    const T D00 = t_fma(Mi01, Ji01, t_fma(Mr01, Jr01, mad2<kSecond>(Mr00, Jr00, Mi00, Ji00)));
+    const T D11 = t_fma(Mi11, Ji11, t_fma(Mr11, Jr11, mad2<kSecond>(Mr10, Jr10, Mi10, Ji10)));
+    const T Dr01 = t_fma(Mi01, Ji11, t_fma(Mr01, Jr11, mad2<kSecond>(Mr00, Jr10, Mi00, Ji10)));
+    const T Di01 = t_fma(-Mr01, Ji11, t_fma(Mi01, Jr11, msb2(Mi00, Jr10, Mr00, Ji10)));
     Y[0] = zn * (D00 + D11);
     Y[1] = zn * (D00 - D11);
     Y[2] = zn * T(2) * Dr01;

@@ -14,26 +14,6 @@ namespace mcrt {
 
 namespace {
 
-template <typename T>
-__device__ __forceinline__ void kext_lookup(const TablesDev& t, T cos_tp, T& a1, T& a2, T& a3) {
-    if (t.k_const) {
-        const float4 k = t.kext[0];
-        a1 = k.x;
-        a2 = k.y;
-        a3 = k.z;
-        return;
-    }
-    const T c = cos_tp > T(1) ? T(1) : (cos_tp < T(-1) ? T(-1) : cos_tp);
-    const T x = t_acos(c) * T(0.31830988618379067) * T(t.n_ktheta - 1);
-    int j = (int)floor(x);
-    j = j > t.n_ktheta - 2 ? t.n_ktheta - 2 : (j < 0 ? 0 : j);
-    const T f = x - T(j);
-    const float4 k0 = t.kext[j], k1 = t.kext[j + 1];
-    a1 = (T(1) - f) * T(k0.x) + f * T(k1.x);
-    a2 = (T(1) - f) * T(k0.y) + f * T(k1.y);
-    a3 = (T(1) - f) * T(k0.z) + f * T(k1.z);
-}
-
 template <typename T> __global__ void __launch_bounds__(128) k_image(const __grid_constant__ ImageParams P) {
     const int nx = P.npix[0], ny = P.npix[1];
     const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -131,10 +111,10 @@ template <typename T> __global__ void __launch_bounds__(128) k_image(const __gri
                     a3 = T(0);
                 } else {
                     const float4 q = P.g.cells[2 * c];
-                    const GrainFrame<T> f = grain_frame(q, Om, phc);
+                    const GrainFrame<T> f = grain_frame<kSecond>(q, Om, phc);
                     c2 = f.c2;
                     s2 = f.s2;
-                    kext_lookup(P.t, f.cos_tp, a1, a2, a3);
+                    kext_eval(P.t, P.t.kext, f.cos_tp, a1, a2, a3);
                 }
                 const T B = T(r.z);
                 // emission: the absorption part of K acting on (B, 0, 0, 0)
@@ -150,8 +130,8 @@ template <typename T> __global__ void __launch_bounds__(128) k_image(const __gri
                     S[3] += f * T(Sc[3]);
                 }
                 rotate_qu(X[1], X[2], c2, s2);
-                cell_step(X, a1, a2, a3, S, kext * ell);
-                rotate_qu(X[1], X[2], c2, -s2);
+                cell_step(cell_coeffs(a1, a2, a3, S, kext * ell), X);
+                rotate_back(X[1], X[2], c2, s2);
             }
             if (lvl == 0) {
                 if (!cross_face(g, idx, p, dir, ell, axis)) break;
@@ -395,7 +375,7 @@ template <typename T> __global__ void k_unit(int fn, long long n, const double* 
         const double* a = in + 12 * i;
         T X[4] = {T(a[0]), T(a[1]), T(a[2]), T(a[3])};
         const T S[4] = {T(a[7]), T(a[8]), T(a[9]), T(a[10])};
-        cell_step(X, T(a[4]), T(a[5]), T(a[6]), S, T(a[11]));
+        cell_step(cell_coeffs(T(a[4]), T(a[5]), T(a[6]), S, T(a[11])), X);
         for (int e = 0; e < 4; ++e) out[4 * i + e] = X[e];
     } else if (fn == 4) {
         const double* a = in + 8 * i;

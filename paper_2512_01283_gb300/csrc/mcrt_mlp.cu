@@ -98,7 +98,7 @@ __device__ void surrogate_label(const LabelTables& T, const V3<float>& ni, const
                         fb * T.bins[((size_t)k1 * T.n_theta + j) * 2].x;
         N = fmaxf(N, v);
     }
-    const float mu = fminf(fmaxf(dot(ni, ns), -1.f), 1.f);
+    const float mu = fminf(fmaxf(dot<kFree>(ni, ns), -1.f), 1.f);
     const float x = acosf(mu) * 0.31830988618379067f * (float)(T.n_theta - 1);
     int j = (int)floorf(x);
     j = j > T.n_theta - 2 ? T.n_theta - 2 : (j < 0 ? 0 : j);

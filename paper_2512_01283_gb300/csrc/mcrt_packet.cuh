@@ -39,7 +39,7 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // alpha1..3 at cos(theta'), linear in theta' on the table grid
-template <typename T>
+template <Fuse F = kSecond, typename T>
 __device__ __forceinline__ void kext_eval(const TablesDev& t, const float4* kx, T cos_tp, T& a1, T& a2, T& a3) {
     if (t.k_const) {
         const float4 k = kx[0];
@@ -54,25 +54,26 @@ __device__ __forceinline__ void kext_eval(const TablesDev& t, const float4* kx, 
     j = j > t.n_ktheta - 2 ? t.n_ktheta - 2 : (j < 0 ? 0 : j);
     const T f = x - T(j);
     const float4 k0 = kx[j], k1 = kx[j + 1];
-    a1 = (T(1) - f) * T(k0.x) + f * T(k1.x);
-    a2 = (T(1) - f) * T(k0.y) + f * T(k1.y);
-    a3 = (T(1) - f) * T(k0.z) + f * T(k1.z);
+    a1 = mad2<F>(T(1) - f, T(k0.x), f, T(k1.x));
+    a2 = mad2<F>(T(1) - f, T(k0.y), f, T(k1.y));
+    a3 = mad2<F>(T(1) - f, T(k0.z), f, T(k1.z));
 }
 
 // scattering matrix of a table (rows of two float4) at mu, linear in the angle
-template <typename T> __device__ __forceinline__ void table_matrix(const float4* tab, int n_theta, T mu, T P[6]) {
+template <Fuse F = kSecond, typename T>
+__device__ __forceinline__ void table_matrix(const float4* tab, int n_theta, T mu, T P[6]) {
     const T c = mu > T(1) ? T(1) : (mu < T(-1) ? T(-1) : mu);
     const T x = t_acos(c) * T(0.31830988618379067) * T(n_theta - 1);
     int j = (int)floor(x);
     j = j > n_theta - 2 ? n_theta - 2 : (j < 0 ? 0 : j);
     const T f = x - T(j), g = T(1) - f;
     const float4 a0 = tab[2 * j], a1 = tab[2 * j + 1], b0 = tab[2 * j + 2], b1 = tab[2 * j + 3];
-    P[0] = g * T(a0.x) + f * T(b0.x);
-    P[1] = g * T(a0.y) + f * T(b0.y);
-    P[2] = g * T(a0.z) + f * T(b0.z);
-    P[3] = g * T(a0.w) + f * T(b0.w);
-    P[4] = g * T(a1.x) + f * T(b1.x);
-    P[5] = g * T(a1.y) + f * T(b1.y);
+    P[0] = mad2<F>(g, T(a0.x), f, T(b0.x));
+    P[1] = mad2<F>(g, T(a0.y), f, T(b0.y));
+    P[2] = mad2<F>(g, T(a0.z), f, T(b0.z));
+    P[3] = mad2<F>(g, T(a0.w), f, T(b0.w));
+    P[4] = mad2<F>(g, T(a1.x), f, T(b1.x));
+    P[5] = mad2<F>(g, T(a1.y), f, T(b1.y));
 }
 
 // Packet state, held in registers for the packet's lifetime (scalar fields only,
@@ -208,10 +209,10 @@ __device__ __forceinline__ void table_at(const TablesDev& t, float s, float mu, 
         k = k > t.n_bins - 2 ? t.n_bins - 2 : (k < 0 ? 0 : k);
         f = x - (float)k;
     }
-    table_matrix(t.bins + (size_t)k * t.n_theta * 2, t.n_theta, mu, P);
+    table_matrix<kFree>(t.bins + (size_t)k * t.n_theta * 2, t.n_theta, mu, P);
     if (f > 0.f) {
         float P2[6];
-        table_matrix(t.bins + (size_t)(k + 1) * t.n_theta * 2, t.n_theta, mu, P2);
+        table_matrix<kFree>(t.bins + (size_t)(k + 1) * t.n_theta * 2, t.n_theta, mu, P2);
 #pragma unroll
         for (int e = 0; e < 6; ++e) P[e] = (1.f - f) * P[e] + f * P2[e];
     }

@@ -352,12 +352,12 @@ __device__ bool emit(const TransportParams& P, const JobRef<T, B>& job, long lon
                      f.cos_tp, a1, a2, s11, s12);
             a3 = T(0);
         } else {
-            kext_eval(tb, job.kext(), f.cos_tp, a1, a2, a3);
+            kext_eval<B ? kFirst : kSecond>(tb, job.kext(), f.cos_tp, a1, a2, a3);
         }
         const T w = (a1 - s11) / (T(tb.alpha1_mean) - omega);
         pk.X0 = eps * w;
         pk.X1 = (a1 - s11) > T(0) ? eps * w * (a2 - s12) / (a1 - s11) : T(0);
-        rotate_qu(pk.X1, pk.X2, f.c2, -f.s2);
+        rotate_back(pk.X1, pk.X2, f.c2, f.s2);
     } else {
         T p[3], n[3];
         if (src.type == MCRT_SRC_POINT) {
@@ -518,7 +518,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
         if (kext > T(0)) {
             const V3<T> n0{pk.nx, pk.ny, pk.nz};
             V3<T> th0, ph0;
-            stokes_basis(n0, th0, ph0);
+            stokes_basis<kSecond>(n0, th0, ph0);
             dip_f = grain_frame(pk.cq, n0, ph0);
             T S2 = (T(1) - dip_f.cos_tp) * (T(1) + dip_f.cos_tp);
             S2 = S2 > T(0) ? S2 : T(0);
@@ -561,7 +561,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
 
     const V3<T> n{pk.nx, pk.ny, pk.nz};
     V3<T> th, ph;
-    stokes_basis(n, th, ph);
+    stokes_basis<kSecond>(n, th, ph);
     const int lane = threadIdx.x & 31;
     const unsigned group = peers & actA;  // same-cell lanes that tally
     const int leader = __ffs(group) - 1;
@@ -585,15 +585,15 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
             const GrainFrame<T> f = grain_frame(pk.cq, n, ph);
             c2 = f.c2;
             s2 = f.s2;
-            kext_eval(tabs, job.kext(), f.cos_tp, a1, a2, a3);
+            kext_eval<B ? kFirst : kSecond>(tabs, job.kext(), f.cos_tp, a1, a2, a3);
         }
         const T a = a1 - omega;
         const T dtau = kext * ell;
         T Xg[4] = {pk.X0, pk.X1, pk.X2, pk.X3};
-        rotate_qu(Xg[1], Xg[2], c2, s2);
+        rotate_qu<SCAT == MCRT_SCAT_DIPOLE ? kSecond : kFirst>(Xg[1], Xg[2], c2, s2);
         T Yg[4], Wg[4];
-        transfer(Xg, a, a2, a3, dtau, Yg, Wg, want_S || SCAT == MCRT_SCAT_DIPOLE, ell);
-        rotate_qu(Yg[1], Yg[2], c2, -s2);
+        transfer<SCAT == kScatTableDeferred>(Xg, a, a2, a3, dtau, Yg, Wg, want_S || SCAT == MCRT_SCAT_DIPOLE, ell);
+        rotate_back(Yg[1], Yg[2], c2, s2);
         // absorbed energy, one FP64 atomic per same-cell group
         {
             const unsigned gmax = kGroups ? __reduce_max_sync(actA, (unsigned)__popc(group)) : 1u;
@@ -603,7 +603,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
             // spheroids the decrease of I also holds kappa_ext s12 int Q dl, which the scattering
             // weight returns in expectation, hence a2 - s12.
             T dI = pk.X0 - Yg[0];
-            if (want_S || SCAT == MCRT_SCAT_DIPOLE) dI = kext * (a * Wg[0] + (a2 - s12) * Wg[1]);
+            if (want_S || SCAT == MCRT_SCAT_DIPOLE) dI = kext * mad2(a, Wg[0], a2 - s12, Wg[1]);
             pk.e_abs += dI;
             if (dI != T(0)) pk.n_abs++;
             if (gmax > 1u) dI = group_sum(actA, group, dI, gmax);
@@ -617,7 +617,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
                 // consecutive slots; a warp that would run past the queue's end writes
                 // empty records and tallies in place below
                 T Wl1 = Wg[1], Wl2 = Wg[2];  // path integral in the packet's basis
-                rotate_qu(Wl1, Wl2, c2, -s2);
+                rotate_back(Wl1, Wl2, c2, s2);
                 const int lead = __ffs(actS) - 1;
                 const unsigned cnt = (unsigned)__popc(actS);
                 unsigned long long base = 0;
@@ -689,7 +689,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
         // the table rounds keep no in-place tally (smaller kernel): a segment that finds
         // no queue space is counted and fails the launch, which the soft limit rules out
         if (SCAT != kScatTableDeferred && want_S && !queued) {
-            rotate_qu(Wg[1], Wg[2], c2, -s2);
+            rotate_back(Wg[1], Wg[2], c2, s2);
             const unsigned gmax = kGroups ? __reduce_max_sync(actS, (unsigned)__popc(group)) : 1u;
             pk.n_tally++;
             double* Sc = job.S() + (size_t)c32 * (size_t)P.n_cam * 4;
@@ -866,12 +866,13 @@ __device__ __forceinline__ bool table_trial(const TablesDev& tabs, int bin, cons
     sn = sn > T(0) ? t_sqrt(sn) : T(0);
     T sa, ca;
     t_sincospi(T(2) * ut.c, &sa, &ca);
-    n2 = V3<T>{mu * n.x + sn * (ca * th.x + sa * ph.x), mu * n.y + sn * (ca * th.y + sa * ph.y),
-               mu * n.z + sn * (ca * th.z + sa * ph.z)};
+    n2 = V3<T>{mad2(mu, n.x, sn, mad2<kSecond>(ca, th.x, sa, ph.x)),
+               mad2(mu, n.y, sn, mad2<kSecond>(ca, th.y, sa, ph.y)),
+               mad2(mu, n.z, sn, mad2<kSecond>(ca, th.z, sa, ph.z))};
     table_matrix(tab, tabs.n_theta, mu, Pm);
     const T bound = ut.d * T(2) * T(tabs.env[c0i + j]) * X[0];
     const T Qs = plane_Q(th, ph, n2, X);
-    return bound < Pm[0] * X[0] + Pm[1] * Qs;
+    return bound < mad2(Pm[0], X[0], Pm[1], Qs);
 }
 
 // Scattering of a packet at its current position (Sec. 2.2): roulette, size bin, then
@@ -883,7 +884,7 @@ __device__ __forceinline__ void scatter_event(const TransportParams& P, const Sm
     const TablesDev& tabs = job.t();
     const V3<T> n{pk.nx, pk.ny, pk.nz};
     V3<T> th, ph;
-    stokes_basis(n, th, ph);
+    stokes_basis<kSecond>(n, th, ph);
     const Draw4<T> us = draw4<T>(pk.pid, pk.n_sca, 0u, P.seed, job.stream());
     if (!roulette(P, pk, us.b, bt)) {
         alive = false;
@@ -915,7 +916,7 @@ __device__ __forceinline__ void scatter_event(const TransportParams& P, const Sm
             n2 = quat_to_lab(pk.cq, V3<T>{g2[0], g2[1], g2[2]});
             V3<T> th2, ph2;
             stokes_basis(n2, th2, ph2);
-            dipole_apply(rho_re, rho_im, zn, ax, th, ph, th2, ph2, X, Y);
+            dipole_apply<kSecond>(rho_re, rho_im, zn, ax, th, ph, th2, ph2, X, Y);
             if (ut.c * env * X[0] < Y[0]) {
                 accepted = true;
                 break;
@@ -953,7 +954,7 @@ __device__ __forceinline__ void scatter_event(const TransportParams& P, const Sm
             rayleigh_matrix(dot(n, n2), Pm);
             const T bound = ut.c * T(2) * T(0.11936620731892133) * X[0];  // 2 * 3/(8 pi)
             const T Qs = plane_Q(th, ph, n2, X);
-            acc = bound < Pm[0] * X[0] + Pm[1] * Qs;
+            acc = bound < mad2<kSecond>(Pm[0], X[0], Pm[1], Qs);
         } else {
             T mu;
             acc = table_trial(tabs, bin, ut, n, th, ph, X, n2, mu, Pm);
@@ -970,9 +971,9 @@ __device__ __forceinline__ void scatter_event(const TransportParams& P, const Sm
     }
     V3<T> th2, ph2;
     stokes_basis(n2, th2, ph2);
-    const PlaneRot<T> pr = plane_rotation(n, th, ph, n2, th2, ph2);
+    const PlaneRot<T> pr = plane_rotation<kFirst, kFirst, kSecond>(n, th, ph, n2, th2, ph2);
     T Y[4];
-    apply_plane(pr, Pm, X, Y);
+    apply_plane<kFirst, kSecond>(pr, Pm, X, Y);
     const T norm = X[0] / Y[0];
     pk.X0 = Y[0] * norm;
     pk.X1 = Y[1] * norm;
@@ -1094,11 +1095,11 @@ __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Sme
     const TablesDev& tabs = job_of<T, B>(P, sm, pk).t();
     const V3<T> n{pk.nx, pk.ny, pk.nz};
     V3<T> th, ph, th2, ph2;
-    stokes_basis(n, th, ph);
+    stokes_basis<kSecond>(n, th, ph);
     stokes_basis(n2a, th2, ph2);
     T Pm[6];
     table_matrix(tabs.bins + (size_t)bin * tabs.n_theta * 2, tabs.n_theta, mua, Pm);
-    const PlaneRot<T> pr = plane_rotation(n, th, ph, n2a, th2, ph2);
+    const PlaneRot<T> pr = plane_rotation<kFirst, kSecond, kSecond>(n, th, ph, n2a, th2, ph2);
     const T X[4] = {pk.X0, pk.X1, pk.X2, pk.X3};
     T Y[4];
     apply_plane(pr, Pm, X, Y);

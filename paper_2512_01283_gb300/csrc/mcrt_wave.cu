@@ -163,13 +163,13 @@ __global__ void __launch_bounds__(kWaveBlock, 1) k_sur_tally(const __grid_consta
                     W[2] = r1.z;
                     W[3] = r1.w;
                     V3<float> th, ph, Om, thc, phc;
-                    stokes_basis(n, th, ph);
+                    stokes_basis<kFree>(n, th, ph);
                     load_camera(s_cam + 12 * cam, Om, thc, phc);
                     // scattering plane of n -> Omega_c, in the lab frame (as the table path)
-                    pr = plane_rotation(n, th, ph, Om, thc, phc);
-                    mu = dot(n, Om);
+                    pr = plane_rotation<kFree>(n, th, ph, Om, thc, phc);
+                    mu = dot<kFree>(n, Om);
                     // the network sees both directions in the grain frame
-                    const V3<float> nGF = quat_to_grain(q, n), cGF = quat_to_grain(q, Om);
+                    const V3<float> nGF = quat_to_grain<kFree>(q, n), cGF = quat_to_grain<kFree>(q, Om);
                     u[0] = nGF.x;
                     u[1] = nGF.y;
                     u[2] = nGF.z;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kWaveBlock, 1) k_sur_tally(const __grid_consta
             } else {
                 float Pm[6];
                 table_at(P.t, s, mu, Pm);
-                apply_plane(pr, Pm, W, Y);
+                apply_plane<kFree>(pr, Pm, W, Y);
                 if (fb)
                     ++c_map;
                 else
@@ -291,11 +291,11 @@ __global__ void __launch_bounds__(tc::kRows * kTcGroups, 1) k_sur_tally_tc(const
                 W[2] = r1.z;
                 W[3] = r1.w;
                 V3<float> th, ph, Om, thc, phc;
-                stokes_basis(n, th, ph);
+                stokes_basis<kFree>(n, th, ph);
                 load_camera(s_cam + 12 * cam, Om, thc, phc);
-                pr = plane_rotation(n, th, ph, Om, thc, phc);
-                mu = dot(n, Om);
-                const V3<float> nGF = quat_to_grain(q, n), cGF = quat_to_grain(q, Om);
+                pr = plane_rotation<kFree>(n, th, ph, Om, thc, phc);
+                mu = dot<kFree>(n, Om);
+                const V3<float> nGF = quat_to_grain<kFree>(q, n), cGF = quat_to_grain<kFree>(q, Om);
                 u[0] = nGF.x;
                 u[1] = nGF.y;
                 u[2] = nGF.z;
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(tc::kRows * kTcGroups, 1) k_sur_tally_tc(const
             } else {
                 float Pm[6];
                 table_at(P.t, s, mu, Pm);
-                apply_plane(pr, Pm, W, Y);
+                apply_plane<kFree>(pr, Pm, W, Y);
                 if (fb)
                     ++c_map;
                 else
@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(kWaveBlock, 1) k_sur_scatter(const __grid_cons
                 const long long c = ((long long)pk.iz * P.g.n[1] + pk.iy) * P.g.n[0] + pk.ix;
                 q = __ldg(&P.g.cells[2 * c]);
                 n = V3<float>{pk.nx, pk.ny, pk.nz};
-                stokes_basis(n, th, ph);
-                nGF = quat_to_grain(q, n);
+                stokes_basis<kFree>(n, th, ph);
+                nGF = quat_to_grain<kFree>(q, n);
             }
         }
         const unsigned pid_lo = (unsigned)((unsigned long long)pk.pid & 0xffffffffull);
@@ -498,10 +498,10 @@ __global__ void __launch_bounds__(kWaveBlock, 1) k_sur_scatter(const __grid_cons
                     bmax = 2.f * tabs.env[(size_t)obin * nint + lo] * oX0 * widen_env;
                     bound = ut.d * bmax;
                     V3<float> th2, ph2;
-                    stokes_basis(n2, th2, ph2);
-                    pr = plane_rotation(V3<float>{onx, ony, onz}, V3<float>{otx, oty, otz}, V3<float>{opx, opy, opz},
+                    stokes_basis<kFree>(n2, th2, ph2);
+                    pr = plane_rotation<kFree>(V3<float>{onx, ony, onz}, V3<float>{otx, oty, otz}, V3<float>{opx, opy, opz},
                                         n2, th2, ph2);
-                    const V3<float> n2GF = quat_to_grain(oq, n2);
+                    const V3<float> n2GF = quat_to_grain<kFree>(oq, n2);
                     u[0] = og.x;
                     u[1] = og.y;
                     u[2] = og.z;
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(kWaveBlock, 1) k_sur_scatter(const __grid_cons
                 } else {
                     float Pm[6];
                     table_at(tabs, osk, mu, Pm);
-                    apply_plane(pr, Pm, oX, Yr);
+                    apply_plane<kFree>(pr, Pm, oX, Yr);
                     if (fb)
                         ++c_map;
                     else
@@ -716,8 +716,8 @@ __global__ void __launch_bounds__(tc::kRows * kScatGroups, 1) k_sur_scatter_tc(c
                     const float4 q = __ldg(&P.g.cells[2 * c]);
                     const V3<float> n{pk.nx, pk.ny, pk.nz};
                     V3<float> th, ph;
-                    stokes_basis(n, th, ph);
-                    const V3<float> gf = quat_to_grain(q, n);
+                    stokes_basis<kFree>(n, th, ph);
+                    const V3<float> gf = quat_to_grain<kFree>(q, n);
                     sp.n[0] = n.x; sp.n[1] = n.y; sp.n[2] = n.z;
                     sp.th[0] = th.x; sp.th[1] = th.y; sp.th[2] = th.z;
                     sp.ph[0] = ph.x; sp.ph[1] = ph.y; sp.ph[2] = ph.z;
@@ -790,10 +790,10 @@ __global__ void __launch_bounds__(tc::kRows * kScatGroups, 1) k_sur_scatter_tc(c
                 bmax = 2.f * tabs.env[(size_t)o.bin * nint + lo] * o.X[0] * widen_env;
                 bound = ut.d * bmax;
                 V3<float> th2, ph2;
-                stokes_basis(n2, th2, ph2);
-                pr = plane_rotation(on, oth, oph, n2, th2, ph2);
+                stokes_basis<kFree>(n2, th2, ph2);
+                pr = plane_rotation<kFree>(on, oth, oph, n2, th2, ph2);
                 const V3<float> og{o.g[0], o.g[1], o.g[2]};
-                const V3<float> n2GF = quat_to_grain(o.q, n2);
+                const V3<float> n2GF = quat_to_grain<kFree>(o.q, n2);
                 u[0] = og.x;
                 u[1] = og.y;
                 u[2] = og.z;
@@ -824,7 +824,7 @@ __global__ void __launch_bounds__(tc::kRows * kScatGroups, 1) k_sur_scatter_tc(c
                 } else {
                     float Pm[6];
                     table_at(tabs, o.sk, mu, Pm);
-                    apply_plane(pr, Pm, oX, r.Y);
+                    apply_plane<kFree>(pr, Pm, oX, r.Y);
                     if (fb)
                         ++c_map;
                     else
