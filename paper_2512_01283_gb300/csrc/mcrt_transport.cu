@@ -9,9 +9,9 @@
 // (DDA), applies the in-cell analytic extinction (App. A) in the grain-meridian basis
 // (eq. rotation-angle / stokes-rotation, quaternions of eq. grain-quaternion), adds
 // its absorbed energy with one FP64 atomic, and tallies the segment's path integral
-// through Z(Omega_cam; Omega_pp) for every camera (eq. scat-disc-sum): in place, one
-// FP64 bulk reduction of the cell's camera rows per lane, or (table rounds and the
-// surrogate) as a record that a tally kernel of its own adds.  Scatterings draw a new
+// through Z(Omega_cam; Omega_pp) for every camera (eq. scat-disc-sum): in place, the warp's
+// staged camera rows as coalesced FP64 reductions, or (table rounds and the surrogate) as a
+// record that a tally kernel of its own adds.  Scatterings draw a new
 // direction by rejection sampling of the polarization-aware cross section, for the
 // warp's waiting lanes together.  Per-step arithmetic runs in T (float or double);
 // the remaining scattering optical depth and all tallies are FP64.
@@ -56,17 +56,21 @@ constexpr int kDefaultBlock = 128;
 template <bool B, int SCAT> constexpr int scatter_batch() {
     return B ? MCRT_SCATTER_BATCH_JOBS : (SCAT == kScatTableDeferred ? MCRT_SCATTER_BATCH_ROUNDS : MCRT_SCATTER_BATCH);
 }
-// per-thread staging slot for the TMA bulk reduction of one segment's source
-// contributions: up to 8 cameras x 4 Stokes FP64 (256 B), padded to 272 B so that
-// the 16-byte stores of a warp spread over all shared-memory banks
-constexpr int kStageCams = 8;
-constexpr int kStageDoubles = 34;
+// in-place tally: a warp's segments stage their cameras' contributions, one row per segment
+// (4 values per camera, the stride an odd number of 16-byte groups, so that the lanes'
+// 16-byte stores fall in different bank groups), beside the rows' addresses
+__host__ __device__ constexpr int stage_row(int n_cam, int value_bytes) {  // in 16-byte groups
+    return (n_cam * value_bytes / 4) | 1;
+}
+__host__ __device__ constexpr int stage_warp_bytes(int n_cam, int value_bytes) {
+    return 32 * (stage_row(n_cam, value_bytes) * 16 + 8);
+}
 
 template <typename T> struct Smem {
     const T* cam;        // [n_cam][12]: Omega, theta-hat, phi-hat (each padded to 4)
     const float4* mix;   // [n_theta][2]
     const float4* kext;  // [n_ktheta]
-    double* stage;       // [blockDim][kStageDoubles]
+    unsigned char* stage;  // this warp's rows, then their addresses
     unsigned long long* chunk;  // round-based paths: per warp, next and end of its record slots
 };
 
@@ -85,6 +89,14 @@ constexpr unsigned kRecChunk = 32u * MCRT_REC_CHUNK;
 #ifndef MCRT_INPLACE_GROUPS
 #define MCRT_INPLACE_GROUPS 0
 #endif
+
+__device__ __forceinline__ void store4(float* d, const float v[4]) {
+    *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store4(double* d, const double v[4]) {
+    reinterpret_cast<double2*>(d)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2*>(d)[1] = make_double2(v[2], v[3]);
+}
 
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
@@ -476,10 +488,11 @@ template <int SCAT> __device__ __forceinline__ void empty_record(const Transport
 }
 
 // One event of a live packet: a cell segment, then a scattering when the sampled
-// optical depth runs out inside the cell.  `work` = live lanes of the warp.
+// optical depth runs out inside the cell.  `work` = live lanes of the warp; `staged` is set
+// to the number of tally rows the warp staged where this lane is one of them.
 template <typename T, int SCAT, bool B, bool R>
 __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm, Packet<T>& pk, bool& alive,
-                                     BlockTotals& bt, unsigned work) {
+                                     BlockTotals& bt, unsigned work, int& staged) {
     const JobRef<T, B> job = job_of<T, B>(P, sm, pk);
     const TablesDev& tabs = job.t();
     const T ks = T(pk.cr.y);
@@ -607,7 +620,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
             pk.e_abs += dI;
             if (dI != T(0)) pk.n_abs++;
             if (gmax > 1u) dI = group_sum(actA, group, dI, gmax);
-            if (lane == leader && dI != T(0)) atomicAdd(&job.absorbed()[c32], widen(dI));
+            if (lane == leader && dI != T(0)) red_add(&job.absorbed()[c32], widen(dI));
         }
         bool queued = false;
         if constexpr (round_based(SCAT)) {
@@ -693,41 +706,36 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
             const unsigned gmax = kGroups ? __reduce_max_sync(actS, (unsigned)__popc(group)) : 1u;
             pk.n_tally++;
             double* Sc = job.S() + (size_t)c32 * (size_t)P.n_cam * 4;
-            double* slot = sm.stage + threadIdx.x * kStageDoubles;
+            const int stride = stage_row(P.n_cam, (int)sizeof(T)) * (16 / (int)sizeof(T));
+            const int rank = __popc(actS & ((1u << lane) - 1u));
+            T* const rows = reinterpret_cast<T*>(sm.stage);
+            T* const row = rows + rank * stride;
+            staged = __popc(actS);
+            reinterpret_cast<double**>(rows + 32 * stride)[rank] = lane == leader ? Sc : nullptr;
             V3<T> ax{T(0), T(0), T(1)};
             if constexpr (SCAT == MCRT_SCAT_DIPOLE) ax = quat_to_lab(pk.cq, ax);
-            for (int k0 = 0; k0 < P.n_cam; k0 += kStageCams) {
-                const int kn = P.n_cam - k0 < kStageCams ? P.n_cam - k0 : kStageCams;
-                if (lane == leader) bulk_wait_read();  // the slot's previous reduction has read it
-                for (int k = 0; k < kn; ++k) {
-                    V3<T> Om, thc, phc;
-                    load_camera(sm.cam + 12 * (k0 + k), Om, thc, phc);
-                    T sv[4];
-                    if constexpr (SCAT == MCRT_SCAT_DIPOLE) {
-                        const DipoleConst<T> dc = dipole_const<T>(tabs.dip);
-                        dipole_apply(dc.rho_re, dc.rho_im, dc.zn, ax, th, ph, thc, phc, Wg,
-                                     sv);
-                    } else {
-                        const T mu = dot(n, Om);
-                        T Pm[6];
-                        if (SCAT == MCRT_SCAT_RAYLEIGH)
-                            rayleigh_matrix(mu, Pm);
-                        else
-                            table_matrix(job.mix(), tabs.n_theta, mu, Pm);
-                        const PlaneRot<T> pr = plane_rotation(n, th, ph, Om, thc, phc);
-                        apply_plane(pr, Pm, Wg, sv);
-                    }
-                    if (gmax > 1u) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) sv[e] = group_sum(actS, group, sv[e], gmax);
-                    }
-                    if (lane == leader) {
-                        double2* d2 = reinterpret_cast<double2*>(slot + 4 * k);
-                        d2[0] = make_double2(widen(sv[0]), widen(sv[1]));
-                        d2[1] = make_double2(widen(sv[2]), widen(sv[3]));
-                    }
+            for (int k = 0; k < P.n_cam; ++k) {
+                V3<T> Om, thc, phc;
+                load_camera(sm.cam + 12 * k, Om, thc, phc);
+                T sv[4];
+                if constexpr (SCAT == MCRT_SCAT_DIPOLE) {
+                    const DipoleConst<T> dc = dipole_const<T>(tabs.dip);
+                    dipole_apply(dc.rho_re, dc.rho_im, dc.zn, ax, th, ph, thc, phc, Wg, sv);
+                } else {
+                    const T mu = dot(n, Om);
+                    T Pm[6];
+                    if (SCAT == MCRT_SCAT_RAYLEIGH)
+                        rayleigh_matrix(mu, Pm);
+                    else
+                        table_matrix(job.mix(), tabs.n_theta, mu, Pm);
+                    const PlaneRot<T> pr = plane_rotation(n, th, ph, Om, thc, phc);
+                    apply_plane(pr, Pm, Wg, sv);
                 }
-                if (lane == leader) bulk_reduce_add_f64(Sc + 4 * k0, slot, (unsigned)kn * 32u);
+                if (gmax > 1u) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) sv[e] = group_sum(actS, group, sv[e], gmax);
+                }
+                store4(row + 4 * k, sv);
             }
         }
         pk.X0 = Yg[0];
@@ -866,8 +874,7 @@ __device__ __forceinline__ bool table_trial(const TablesDev& tabs, int bin, cons
     sn = sn > T(0) ? t_sqrt(sn) : T(0);
     T sa, ca;
     t_sincospi(T(2) * ut.c, &sa, &ca);
-    n2 = V3<T>{mad2(mu, n.x, sn, mad2<kSecond>(ca, th.x, sa, ph.x)),
-               mad2(mu, n.y, sn, mad2<kSecond>(ca, th.y, sa, ph.y)),
+    n2 = V3<T>{mad2(mu, n.x, sn, mad2<kSecond>(ca, th.x, sa, ph.x)), mad2(mu, n.y, sn, mad2<kSecond>(ca, th.y, sa, ph.y)),
                mad2(mu, n.z, sn, mad2<kSecond>(ca, th.z, sa, ph.z))};
     table_matrix(tab, tabs.n_theta, mu, Pm);
     const T bound = ut.d * T(2) * T(tabs.env[c0i + j]) * X[0];
@@ -1151,7 +1158,8 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
     const int n_mix = (!B && SCAT != MCRT_SCAT_RAYLEIGH && SCAT != MCRT_SCAT_DIPOLE) ? 2 * P.t.n_theta : 0;
     T* s_cam = reinterpret_cast<T*>(s_mix + n_mix);
     const int cam_bytes = 12 * P.n_cam * (int)sizeof(T);
-    double* s_stage = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(s_cam) + cam_bytes);
+    unsigned char* s_stage = reinterpret_cast<unsigned char*>(s_cam) + cam_bytes +
+                             (threadIdx.x >> 5) * stage_warp_bytes(P.n_cam, (int)sizeof(T));
     for (int i = threadIdx.x; i < n_k; i += blockDim.x) s_kext[i] = P.t.kext[i];
     for (int i = threadIdx.x; i < n_mix; i += blockDim.x) s_mix[i] = P.t.mix[i];
     for (int i = threadIdx.x; i < 12 * P.n_cam; i += blockDim.x) {
@@ -1161,8 +1169,8 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
     }
     if (threadIdx.x < 6) bt.e[threadIdx.x] = 0.0;
     if (threadIdx.x < 10) bt.n[threadIdx.x] = 0ull;
-    if (threadIdx.x < 2 * (kDefaultBlock / 32)) s_chunk[threadIdx.x] = 0ull;
     if (threadIdx.x == 0) bt.status = 0u;
+    if (threadIdx.x < 2 * (kDefaultBlock / 32)) s_chunk[threadIdx.x] = 0ull;
     __syncthreads();
 
     const Smem<T> sm{s_cam, s_mix, s_kext, s_stage, s_chunk};
@@ -1271,7 +1279,18 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
             }
             continue;
         }
-        if (alive && !pk.pending) step<T, SCAT, B, R>(P, sm, pk, alive, bt, work);
+        int staged = 0;
+        if (alive && !pk.pending) step<T, SCAT, B, R>(P, sm, pk, alive, bt, work, staged);
+        if constexpr (!round_based(SCAT)) {
+            const int rows = __reduce_max_sync(kFull, staged);
+            if (rows > 0) {
+                const int stride = stage_row(P.n_cam, (int)sizeof(T)) * (16 / (int)sizeof(T));
+                const T* const r = reinterpret_cast<const T*>(s_stage);
+                double* const* const at = reinterpret_cast<double* const*>(r + 32 * stride);
+                reduce_rows(rows, threadIdx.x & 31, r, stride, 4 * P.n_cam, [&](int k) { return at[k]; });
+                __syncwarp();
+            }
+        }
     }
 
     if constexpr (round_based(SCAT) && kRecChunk > 0) {
@@ -1281,7 +1300,6 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
         for (unsigned long long k = next + (threadIdx.x & 31); k < end && k < P.sur.rec_cap; k += 32)
             empty_record<SCAT>(P, k);
     }
-    bulk_wait_all();  // this thread's reductions have completed before the block ends
     __syncthreads();
     if (threadIdx.x < 6) {
         atomicAdd(&P.stats[threadIdx.x], bt.e[threadIdx.x]);
@@ -1354,7 +1372,9 @@ size_t transport_smem_bytes(const TransportParams& p, int precision, int block) 
     const size_t mix = (!batch && p.t.model == MCRT_SCAT_TABLE) ? 2 * (size_t)p.t.n_theta * sizeof(float4) : 0;
     const size_t cams = 12 * (size_t)p.n_cam * tsize;
     // the table rounds tally in their own kernel: no staging slots
-    const size_t stage = p.sur.deferred == kScatTableDeferred ? 0 : (size_t)block * kStageDoubles * sizeof(double);
+    const size_t stage = p.sur.deferred == kScatTableDeferred || p.n_cam == 0
+                             ? 0
+                             : (size_t)(block / 32) * stage_warp_bytes(p.n_cam, (int)tsize);
     return kx + mix + cams + stage;
 }
 
