@@ -30,7 +30,7 @@ struct mcrt_ctx {
     bool tables_set = false;
     TablesDev t{};
     float4 *d_mix = nullptr, *d_bins = nullptr, *d_kext = nullptr;
-    double *d_env_cdf = nullptr, *d_bin_cdf = nullptr, *d_alpha1 = nullptr;
+    double *d_env_cdf = nullptr, *d_bin_cdf = nullptr, *d_cos = nullptr, *d_alpha1 = nullptr;
     float* d_env = nullptr;
     // thermal emission CDF
     double* d_cdf = nullptr;
@@ -174,10 +174,11 @@ void free_tables(mcrt_ctx* c) {
     cudaFree(c->d_kext);
     cudaFree(c->d_env_cdf);
     cudaFree(c->d_bin_cdf);
+    cudaFree(c->d_cos);
     cudaFree(c->d_alpha1);
     cudaFree(c->d_env);
     c->d_mix = c->d_bins = c->d_kext = nullptr;
-    c->d_env_cdf = c->d_bin_cdf = c->d_alpha1 = nullptr;
+    c->d_env_cdf = c->d_bin_cdf = c->d_cos = c->d_alpha1 = nullptr;
     c->d_env = nullptr;
     c->tables_set = false;
 }
@@ -394,6 +395,7 @@ mcrt_status mcrt_set_dust_tables(mcrt_ctx* ctx, int32_t model, int32_t n_bins, i
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_env_cdf, (size_t)nb * nint * (sizeof(double) + sizeof(float)));
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_env, (size_t)nb * nint * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_bin_cdf, (size_t)nb * (sizeof(double) + sizeof(float)));
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_cos, (size_t)nt * (sizeof(double) + sizeof(float)));
     if (e != cudaSuccess) {
         free_tables(ctx);
         return fail(ctx, MCRT_E_NOMEM, "mcrt_set_dust_tables: %s", cudaGetErrorString(e));
@@ -408,7 +410,7 @@ mcrt_status mcrt_set_dust_tables(mcrt_ctx* ctx, int32_t model, int32_t n_bins, i
         if (e == cudaSuccess)
             e = launch_prepare_tables(model, n_bins, n_theta, n_ktheta, (const float*)dm.ptr, (const float*)dw.ptr,
                                       (const float*)dk.ptr, ctx->d_mix, ctx->d_bins, ctx->d_env_cdf, ctx->d_env,
-                                      ctx->d_bin_cdf, ctx->d_kext, ctx->d_alpha1, ctx->stream);
+                                      ctx->d_bin_cdf, ctx->d_cos, ctx->d_kext, ctx->d_alpha1, ctx->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&a1m, ctx->d_alpha1, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     }
@@ -430,6 +432,8 @@ mcrt_status mcrt_set_dust_tables(mcrt_ctx* ctx, int32_t model, int32_t n_bins, i
     t.bin_cdf = ctx->d_bin_cdf;
     t.env_cdf_f = reinterpret_cast<const float*>(ctx->d_env_cdf + (size_t)nb * nint);
     t.bin_cdf_f = reinterpret_cast<const float*>(ctx->d_bin_cdf + nb);
+    t.cos_d = ctx->d_cos;
+    t.cos_f = reinterpret_cast<const float*>(ctx->d_cos + nt);
     t.kext = ctx->d_kext;
     t.alpha1_mean = a1m;
     ctx->tables_set = true;

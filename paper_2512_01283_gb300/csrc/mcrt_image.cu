@@ -196,12 +196,14 @@ __global__ void k_setup_cells(const float* __restrict__ ka, const float* __restr
 // piecewise-constant envelope of P11 with its normalised cumulative weights,
 // cumulative bin weights, extinction rows and the sphere average of alpha1.  The two
 // cumulative tables are followed by their FP32 copies (env_cdf holds n_bins (n_theta - 1)
-// doubles and as many floats, bin_cdf n_bins doubles and n_bins floats).
+// doubles and as many floats, bin_cdf n_bins doubles and n_bins floats), as are the cosines of
+// the tabulated angles (n_theta doubles, n_theta floats, each the limit of an interval as a
+// trial in that precision would compute it).
 __global__ void k_prepare_tables(int model, int n_bins, int n_theta, int n_ktheta, const float* __restrict__ mueller,
                                  const float* __restrict__ bin_weight, const float* __restrict__ kext,
                                  float4* __restrict__ mix, float4* __restrict__ bins, double* __restrict__ env_cdf,
-                                 float* __restrict__ env, double* __restrict__ bin_cdf, float4* __restrict__ kext4,
-                                 double* __restrict__ alpha1_mean) {
+                                 float* __restrict__ env, double* __restrict__ bin_cdf, double* __restrict__ cosines,
+                                 float4* __restrict__ kext4, double* __restrict__ alpha1_mean) {
     const double pi = 3.141592653589793;
     for (int j = threadIdx.x; j < n_ktheta; j += blockDim.x)
         kext4[j] = make_float4(kext[3 * j], kext[3 * j + 1], kext[3 * j + 2], 0.f);
@@ -258,6 +260,15 @@ __global__ void k_prepare_tables(int model, int n_bins, int n_theta, int n_kthet
     float* bin_cdf_f = reinterpret_cast<float*>(bin_cdf + n_bins);
     for (int i = threadIdx.x; i < n_bins * nint; i += blockDim.x) env_cdf_f[i] = (float)env_cdf[i];
     for (int k = threadIdx.x; k < n_bins; k += blockDim.x) bin_cdf_f[k] = (float)bin_cdf[k];
+    float* cos_f = reinterpret_cast<float*>(cosines + n_theta);
+    for (int j = threadIdx.x; j < n_theta; j += blockDim.x) {
+        double sd, cd;
+        float sf, cf;
+        sincospi((double)j / (double)nint, &sd, &cd);
+        sincospif((float)j / (float)nint, &sf, &cf);
+        cosines[j] = cd;
+        cos_f[j] = cf;
+    }
 }
 
 // Thermal emission weights kappa_ext (mean alpha1 - omega) B V and their inclusive
@@ -537,11 +548,11 @@ cudaError_t launch_setup_cells(const float* ka, const float* ks, const float* bf
 
 cudaError_t launch_prepare_tables(int model, int n_bins, int n_theta, int n_ktheta, const float* mueller,
                                   const float* bin_weight, const float* kext, float4* mix, float4* bins,
-                                  double* env_cdf, float* env, double* bin_cdf, float4* kext4, double* alpha1_mean,
-                                  cudaStream_t s) {
+                                  double* env_cdf, float* env, double* bin_cdf, double* cosines, float4* kext4,
+                                  double* alpha1_mean, cudaStream_t s) {
     (void)cudaGetLastError();  // report this launch's error only
     k_prepare_tables<<<1, 256, 0, s>>>(model, n_bins, n_theta, n_ktheta, mueller, bin_weight, kext, mix, bins,
-                                       env_cdf, env, bin_cdf, kext4, alpha1_mean);
+                                       env_cdf, env, bin_cdf, cosines, kext4, alpha1_mean);
     return cudaGetLastError();
 }
 

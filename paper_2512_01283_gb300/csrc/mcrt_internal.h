@@ -100,15 +100,19 @@ struct TablesDev {
     // the FP32 kernels, which compare in FP32: no FP64 conversion per search step
     const float* env_cdf_f;
     const float* bin_cdf_f;
+    // cos(pi j / (n_theta - 1)) of the tabulated angles, in FP64 and in FP32 (each computed in its
+    // own precision): the limits of the envelope's intervals
+    const double* cos_d;
+    const float* cos_f;
     const float4* kext;   // [n_ktheta] (alpha1, alpha2, alpha3, 0)
     double alpha1_mean;
     DipoleDev dip;        // MCRT_SCAT_DIPOLE constants
 };
 
-// Entry i of a cumulative weight table in the kernel's arithmetic type.
-template <typename T> __device__ __forceinline__ T cdf_at(const double* d, const float* f, size_t i);
-template <> __device__ __forceinline__ float cdf_at<float>(const double*, const float* f, size_t i) { return f[i]; }
-template <> __device__ __forceinline__ double cdf_at<double>(const double* d, const float*, size_t i) { return d[i]; }
+// Entry i of a table kept in both precisions, in the kernel's arithmetic type.
+template <typename T> __device__ __forceinline__ T entry_at(const double* d, const float* f, size_t i);
+template <> __device__ __forceinline__ float entry_at<float>(const double*, const float* f, size_t i) { return f[i]; }
+template <> __device__ __forceinline__ double entry_at<double>(const double* d, const float*, size_t i) { return d[i]; }
 
 struct SourceDev {
     int type, beam_dir;
@@ -240,8 +244,8 @@ cudaError_t launch_setup_cells(const float* ka, const float* ks, const float* bf
                                float4* cells, unsigned* bad, cudaStream_t s);
 cudaError_t launch_prepare_tables(int model, int n_bins, int n_theta, int n_ktheta, const float* mueller,
                                   const float* bin_weight, const float* kext, float4* mix, float4* bins,
-                                  double* env_cdf, float* env, double* bin_cdf, float4* kext4, double* alpha1_mean,
-                                  cudaStream_t s);
+                                  double* env_cdf, float* env, double* bin_cdf, double* cosines, float4* kext4,
+                                  double* alpha1_mean, cudaStream_t s);
 cudaError_t launch_thermal_cdf(const GridDev& g, double alpha1_mean, double* cdf, double* block_sums, int n_blocks,
                                cudaStream_t s);
 int thermal_cdf_blocks(long long ncell);

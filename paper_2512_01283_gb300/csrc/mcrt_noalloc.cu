@@ -37,7 +37,8 @@ constexpr size_t kOffBins = kOffMix + round256((size_t)kMaxTheta * 2 * sizeof(fl
 constexpr size_t kOffEnvCdf = kOffBins + round256((size_t)kMaxBins * kMaxTheta * 2 * sizeof(float4));
 constexpr size_t kOffEnv = kOffEnvCdf + round256((size_t)kMaxBins * (kMaxTheta - 1) * (sizeof(double) + sizeof(float)));
 constexpr size_t kOffBinCdf = kOffEnv + round256((size_t)kMaxBins * (kMaxTheta - 1) * sizeof(float));
-constexpr size_t kOffKext = kOffBinCdf + round256((size_t)kMaxBins * (sizeof(double) + sizeof(float)));
+constexpr size_t kOffCos = kOffBinCdf + round256((size_t)kMaxBins * (sizeof(double) + sizeof(float)));
+constexpr size_t kOffKext = kOffCos + round256((size_t)kMaxTheta * (sizeof(double) + sizeof(float)));
 constexpr size_t kOffWork = kOffKext + round256((size_t)kMaxTheta * sizeof(float4));
 // work area: packet counter (8 B), 16 totals (128 B), status (8 B), alpha1 mean (8 B),
 // invalid-input flag (8 B)
@@ -181,7 +182,7 @@ extern "C" mcrt_status mcrt_launch_packets_noalloc(const mcrt_noalloc_problem* p
                                 pr->bin_weight, pr->kext, reinterpret_cast<float4*>(base + kOffMix),
                                 reinterpret_cast<float4*>(base + kOffBins), reinterpret_cast<double*>(base + kOffEnvCdf),
                                 reinterpret_cast<float*>(base + kOffEnv), reinterpret_cast<double*>(base + kOffBinCdf),
-                                reinterpret_cast<float4*>(base + kOffKext), reinterpret_cast<double*>(work + 144), s));
+                                reinterpret_cast<double*>(base + kOffCos), reinterpret_cast<float4*>(base + kOffKext), reinterpret_cast<double*>(work + 144), s));
     unsigned bad = 0;
     NA_CK(cudaMemcpyAsync(&bad, work + 152, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     NA_CK(cudaStreamSynchronize(s));
@@ -202,6 +203,8 @@ extern "C" mcrt_status mcrt_launch_packets_noalloc(const mcrt_noalloc_problem* p
     // the FP32 copies follow the FP64 tables (as k_prepare_tables writes them)
     t.env_cdf_f = reinterpret_cast<const float*>(t.env_cdf + (size_t)t.n_bins * (t.n_theta > 1 ? t.n_theta - 1 : 0));
     t.bin_cdf_f = reinterpret_cast<const float*>(t.bin_cdf + t.n_bins);
+    t.cos_d = reinterpret_cast<const double*>(base + kOffCos);
+    t.cos_f = reinterpret_cast<const float*>(t.cos_d + t.n_theta);
     t.kext = reinterpret_cast<const float4*>(base + kOffKext);
     t.alpha1_mean = 1.0;  // used by thermal sources only, which are not accepted here
 

@@ -485,9 +485,7 @@ __global__ void __launch_bounds__(kWaveBlock, 1) k_sur_scatter(const __grid_cons
                         else
                             lo = mid + 1;
                     }
-                    float s0, c0, s1, c1;
-                    sincospif((float)lo / (float)nint, &s0, &c0);
-                    sincospif((float)(lo + 1) / (float)nint, &s1, &c1);
+                    const float c0 = tabs.cos_f[lo], c1 = tabs.cos_f[lo + 1];
                     mu = c0 - ut.b * (c0 - c1);
                     float sn = (1.f - mu) * (1.f + mu);
                     sn = sn > 0.f ? sqrtf(sn) : 0.f;
@@ -777,9 +775,7 @@ __global__ void __launch_bounds__(tc::kRows * kScatGroups, 1) k_sur_scatter_tc(c
                     else
                         lo = mid + 1;
                 }
-                float s0, c0, s1, c1;
-                sincospif((float)lo / (float)nint, &s0, &c0);
-                sincospif((float)(lo + 1) / (float)nint, &s1, &c1);
+                const float c0 = tabs.cos_f[lo], c1 = tabs.cos_f[lo + 1];
                 mu = c0 - ut.b * (c0 - c1);
                 float sn = (1.f - mu) * (1.f + mu);
                 sn = sn > 0.f ? sqrtf(sn) : 0.f;
