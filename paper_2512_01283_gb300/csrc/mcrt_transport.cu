@@ -36,11 +36,20 @@ constexpr int kDefaultBlock = 128;
 #define MCRT_MIN_BLOCKS 5
 #endif
 // lanes of a warp that wait before the warp runs the scattering code (or takes new
-// packets) for all of them at once.  Measured on GB300: the in-place kernels run fastest
-// with 4 and 4; the table rounds of the 192^3 disk, whose births run in a kernel of their
-// own, with 6 scatterings (transport 718 ms per 1e8-packet step, against 728 with 4 and
-// 738 with 3) and 4 resumed packets (752 ms with 1 or 8); the batched launch of the
-// 256-job sweep with 8 and 4 (9.4e9 events/s; 8.7e9 with 4 and 4, 7.5e9 with 1 and 1)
+// packets) for all of them at once; a scattering phase also starts as soon as as many lanes
+// wait as move (at the end of a launch, when no new packets come, waiting for a full group
+// only delayed the last ones).  The more often packets scatter the sooner a larger group is
+// together; what waiting lanes idle meets the phase's cost at these counts, measured on GB300
+// with the trials spread over the warp:
+//   Rayleigh 8: plane-parallel slab (41 scatterings a packet) 405 ms, 431 with 4 and 406 with 10;
+//   spheroids and FP64 tables 4: spheroid sphere (0.6 scatterings a packet) 69.3 ms, 70.0 with 3,
+//     72.3 with 8; FP64 disk of 1e5 packets 12.2 ms, 13.3 with 8;
+//   table rounds 6: transport of 5e6 star and 5e6 thermal packets of the 192^3 disk 42.4 + 24.8 ms,
+//     42.8 + 24.9 with 5 and 42.7 + 24.8 with 8;
+//   batched launches 8 (9.4e9 events/s on the 256-job sweep, 8.7e9 with 4).
+// New packets are taken by 4 lanes together (5: slab 409 ms; singly: batched sweep 7.5e9 events/s
+// against 8.7e9); a rule on the lane steps spent waiting, instead of the counts, came within 3 %
+// on every workload but was better on none.
 #ifndef MCRT_SCATTER_BATCH
 #define MCRT_SCATTER_BATCH 4
 #endif
@@ -50,11 +59,17 @@ constexpr int kDefaultBlock = 128;
 #ifndef MCRT_SCATTER_BATCH_JOBS
 #define MCRT_SCATTER_BATCH_JOBS 8
 #endif
+#ifndef MCRT_SCATTER_BATCH_RAYLEIGH
+#define MCRT_SCATTER_BATCH_RAYLEIGH 8
+#endif
 #ifndef MCRT_REFILL_BATCH
 #define MCRT_REFILL_BATCH 4
 #endif
 template <bool B, int SCAT> constexpr int scatter_batch() {
-    return B ? MCRT_SCATTER_BATCH_JOBS : (SCAT == kScatTableDeferred ? MCRT_SCATTER_BATCH_ROUNDS : MCRT_SCATTER_BATCH);
+    return B ? MCRT_SCATTER_BATCH_JOBS
+             : (SCAT == kScatTableDeferred
+                    ? MCRT_SCATTER_BATCH_ROUNDS
+                    : (SCAT == MCRT_SCAT_RAYLEIGH ? MCRT_SCATTER_BATCH_RAYLEIGH : MCRT_SCATTER_BATCH));
 }
 // in-place tally: a warp's segments stage their cameras' contributions, one row per segment
 // (4 values per camera, the stride an odd number of 16-byte groups, so that the lanes'
@@ -811,7 +826,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
         alive = false;
         return;
     }
-    // the rejection sampling waits until enough lanes of the warp need it (scatter_event)
+    // the rejection sampling waits until enough lanes of the warp need it (scatter_coop)
     pk.pending = true;
 }
 
@@ -883,114 +898,34 @@ __device__ __forceinline__ bool table_trial(const TablesDev& tabs, int bin, cons
     return bound < mad2(Pm[0], X[0], Pm[1], Qs);
 }
 
-// Scattering of a packet at its current position (Sec. 2.2): roulette, size bin, then
-// rejection sampling of the new direction; run for the warp's waiting lanes together.
-template <typename T, int SCAT, bool B>
-__device__ __forceinline__ void scatter_event(const TransportParams& P, const Smem<T>& sm, Packet<T>& pk, bool& alive,
-                                              BlockTotals& bt) {
-    const JobRef<T, B> job = job_of<T, B>(P, sm, pk);
-    const TablesDev& tabs = job.t();
-    const V3<T> n{pk.nx, pk.ny, pk.nz};
-    V3<T> th, ph;
-    stokes_basis<kSecond>(n, th, ph);
-    const Draw4<T> us = draw4<T>(pk.pid, pk.n_sca, 0u, P.seed, job.stream());
-    if (!roulette(P, pk, us.b, bt)) {
-        alive = false;
-        return;
-    }
-    if constexpr (SCAT == MCRT_SCAT_DIPOLE) {
-        // aligned spheroid: isotropic proposal, envelope env I >= (Zhat X)_0; the new
-        // Stokes vector is Zhat X (K_sca X)_0 / (s11 (Zhat X)_0), i.e. Zhat X renormalised
-        // to I + (s12 / s11) Q with Q in the grain-meridian basis
-        const DipoleConst<T> dp = dipole_const<T>(tabs.dip);
-        const V3<T> ax = quat_to_lab(pk.cq, V3<T>{T(0), T(0), T(1)});
-        const GrainFrame<T> f = grain_frame(pk.cq, n, ph);
-        T Qg = pk.X1, Ug = pk.X2;
-        rotate_qu(Qg, Ug, f.c2, f.s2);
-        T S2 = (T(1) - f.cos_tp) * (T(1) + f.cos_tp);
-        S2 = S2 > T(0) ? S2 : T(0);
-        const T hs = (dp.cs1 - dp.cs0) * T(0.5) * S2;
-        const T Iw = pk.X0 + t_div(hs, dp.cs0 + hs) * Qg;
-        const T X[4] = {pk.X0, pk.X1, pk.X2, pk.X3};
-        const T rho_re = dp.rho_re, rho_im = dp.rho_im, zn = dp.zn, env = dp.env;
-        V3<T> n2;
-        T Y[4];
-        bool accepted = false;
-        for (int t = 0; t < P.max_trials; ++t) {
-            const Draw4<T> ut = draw4<T>(pk.pid, pk.n_sca, 1u + (unsigned)t, P.seed, job.stream());
-            pk.trials++;
-            T g2[3];
-            iso_dir(ut.a, ut.b, g2);
-            n2 = quat_to_lab(pk.cq, V3<T>{g2[0], g2[1], g2[2]});
-            V3<T> th2, ph2;
-            stokes_basis(n2, th2, ph2);
-            dipole_apply<kSecond>(rho_re, rho_im, zn, ax, th, ph, th2, ph2, X, Y);
-            if (ut.c * env * X[0] < Y[0]) {
-                accepted = true;
-                break;
-            }
-        }
-        if (!accepted) {
-            finish(P, pk, 4, bt);
-            alive = false;
-            return;
-        }
-        const T norm = Iw / Y[0];
-        pk.X0 = Y[0] * norm;
-        pk.X1 = Y[1] * norm;
-        pk.X2 = Y[2] * norm;
-        pk.X3 = Y[3] * norm;
-        pk.nx = n2.x;
-        pk.ny = n2.y;
-        pk.nz = n2.z;
-        tau_set(pk.tau, -t_log(us.a));
-        return;
-    }
-    const int bin = table_optics(SCAT) ? size_bin(tabs, us.c) : 0;
-    const T X[4] = {pk.X0, pk.X1, pk.X2, pk.X3};
-    V3<T> n2;
+// One trial of the rejection sampling of a dipole (Rayleigh) scattering: isotropic proposal
+// in the grain frame (3 / 4 of the trials' constant is the peak of P11), accepted like a
+// tabulated one.
+template <typename T>
+__device__ __forceinline__ bool rayleigh_trial(const float4& q, const Draw4<T>& ut, const V3<T>& n, const V3<T>& th,
+                                               const V3<T>& ph, const T X[4], V3<T>& n2) {
+    T g2[3];
+    iso_dir(ut.a, ut.b, g2);
+    n2 = quat_to_lab(q, V3<T>{g2[0], g2[1], g2[2]});
     T Pm[6];
-    bool accepted = false;
-    for (int t = 0; t < P.max_trials; ++t) {
-        const Draw4<T> ut = draw4<T>(pk.pid, pk.n_sca, 1u + (unsigned)t, P.seed, job.stream());
-        pk.trials++;
-        bool acc;
-        if (SCAT == MCRT_SCAT_RAYLEIGH) {
-            T g2[3];
-            iso_dir(ut.a, ut.b, g2);
-            n2 = quat_to_lab(pk.cq, V3<T>{g2[0], g2[1], g2[2]});
-            rayleigh_matrix(dot(n, n2), Pm);
-            const T bound = ut.c * T(2) * T(0.11936620731892133) * X[0];  // 2 * 3/(8 pi)
-            const T Qs = plane_Q(th, ph, n2, X);
-            acc = bound < mad2<kSecond>(Pm[0], X[0], Pm[1], Qs);
-        } else {
-            T mu;
-            acc = table_trial(tabs, bin, ut, n, th, ph, X, n2, mu, Pm);
-        }
-        if (acc) {
-            accepted = true;
-            break;
-        }
-    }
-    if (!accepted) {
-        finish(P, pk, 4, bt);
-        alive = false;
-        return;
-    }
+    rayleigh_matrix(dot(n, n2), Pm);
+    const T bound = ut.c * T(2) * T(0.11936620731892133) * X[0];  // 2 * 3/(8 pi)
+    const T Qs = plane_Q(th, ph, n2, X);
+    return bound < mad2<kSecond>(Pm[0], X[0], Pm[1], Qs);
+}
+
+// One trial of an aligned spheroid: isotropic proposal, envelope env I >= (Zhat X)_0.
+template <typename T>
+__device__ __forceinline__ bool dipole_trial(const DipoleConst<T>& dp, const float4& q, const Draw4<T>& ut,
+                                             const V3<T>& th, const V3<T>& ph, const T X[4], V3<T>& n2, T Y[4]) {
+    T g2[3];
+    iso_dir(ut.a, ut.b, g2);
+    n2 = quat_to_lab(q, V3<T>{g2[0], g2[1], g2[2]});
     V3<T> th2, ph2;
     stokes_basis(n2, th2, ph2);
-    const PlaneRot<T> pr = plane_rotation<kFirst, kFirst, kSecond>(n, th, ph, n2, th2, ph2);
-    T Y[4];
-    apply_plane<kFirst, kSecond>(pr, Pm, X, Y);
-    const T norm = X[0] / Y[0];
-    pk.X0 = Y[0] * norm;
-    pk.X1 = Y[1] * norm;
-    pk.X2 = Y[2] * norm;
-    pk.X3 = Y[3] * norm;
-    pk.nx = n2.x;
-    pk.ny = n2.y;
-    pk.nz = n2.z;
-    tau_set(pk.tau, -t_log(us.a));
+    const V3<T> ax = quat_to_lab(q, V3<T>{T(0), T(0), T(1)});
+    dipole_apply<kSecond>(dp.rho_re, dp.rho_im, dp.zn, ax, th, ph, th2, ph2, X, Y);
+    return ut.c * dp.env * X[0] < Y[0];
 }
 
 // Lane of the k-th set bit of m (k < popc(m)), by halving.
@@ -1011,17 +946,23 @@ __device__ __forceinline__ int nth_set_lane(unsigned m, int k) {
     return pos;
 }
 
-// Scatterings of the warp's waiting lanes with their rejection trials spread over all
-// 32 lanes (launches with tabulated optics; in batched launches each trial lane reads
-// the tables of its packet's job).  Each owner first takes its roulette and size bin;
-// then, round after round, every unresolved packet gets floor(32 / unresolved) lanes
-// that evaluate its next trials in trial order, and the packet takes its first
-// accepted trial.  Direction, matrix and trial count are thus those of the sequential
-// rule (same random numbers, same arithmetic; the trial reads I, Q and U only, so V
-// is not passed).  All 32 lanes call it.
-template <typename T, bool B>
+template <typename T> __device__ __forceinline__ V3<T> shfl3(const V3<T>& v, int src) {
+    return V3<T>{__shfl_sync(kFull, v.x, src), __shfl_sync(kFull, v.y, src), __shfl_sync(kFull, v.z, src)};
+}
+
+// Scatterings of the warp's waiting lanes (Sec. 2.2) with their rejection trials spread over
+// all 32 lanes (in batched launches each trial lane reads the tables of its packet's job).
+// Each owner first takes its roulette and size bin; then, round after round, every
+// unresolved packet gets floor(32 / unresolved) lanes that evaluate its next trials in trial
+// order, and the packet takes its first accepted trial.  Direction, matrix and trial count are
+// thus those of the sequential rule (same random numbers, same arithmetic; V is passed
+// where a trial reads it, for aligned spheroids).  All 32 lanes call it.  Measured against
+// every lane looping over its own trials: plane-parallel slab, 1e7 packets, 480 -> 431 ms
+// (groups of 4), spheroids 70.2 -> 69.5 ms.
+template <typename T, int SCAT, bool B>
 __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Smem<T>& sm, Packet<T>& pk, bool& alive,
                                              BlockTotals& bt) {
+    constexpr bool kTable = table_optics(SCAT), kDipole = SCAT == MCRT_SCAT_DIPOLE;
     const int lane = threadIdx.x & 31;
     bool live = false;
     int bin = 0;
@@ -1029,29 +970,33 @@ __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Sme
     if (alive && pk.pending) {
         pk.pending = false;
         const JobRef<T, B> job = job_of<T, B>(P, sm, pk);
-        const TablesDev& tabs = job.t();
         const Draw4<T> us = draw4<T>(pk.pid, pk.n_sca, 0u, P.seed, job.stream());
         live = roulette(P, pk, us.b, bt);
         alive = live;
-        bin = size_bin(tabs, us.c);
+        if constexpr (kTable) bin = size_bin(job.t(), us.c);
         u_tau = us.a;
     }
     unsigned todo = __ballot_sync(kFull, live);
     int t_next = 0;          // owner: first trial of its next round
     bool accepted = false;   // owner: a trial was accepted
     V3<T> n2a{T(0), T(0), T(1)};
-    T mua = T(1);
+    T mua = T(1);            // tables: cosine of the scattering angle
+    T Ya[4] = {T(1), T(0), T(0), T(0)};  // spheroids: Zhat X of the accepted trial
     while (todo != 0u) {
         const int nu = __popc(todo);
         const int per = 32 / nu;
         const int k = lane / per;  // packet this lane evaluates (rank among the unresolved)
         const int src = k < nu ? nth_set_lane(todo, k) : lane;
-        const V3<T> n{__shfl_sync(kFull, pk.nx, src), __shfl_sync(kFull, pk.ny, src), __shfl_sync(kFull, pk.nz, src)};
-        const T X[4] = {__shfl_sync(kFull, pk.X0, src), __shfl_sync(kFull, pk.X1, src),
-                        __shfl_sync(kFull, pk.X2, src), T(0)};
+        const V3<T> n = shfl3(V3<T>{pk.nx, pk.ny, pk.nz}, src);
+        T X[4] = {__shfl_sync(kFull, pk.X0, src), __shfl_sync(kFull, pk.X1, src), __shfl_sync(kFull, pk.X2, src), T(0)};
+        float4 q = pk.cq;
+        if constexpr (!kTable)
+            q = make_float4(__shfl_sync(kFull, pk.cq.x, src), __shfl_sync(kFull, pk.cq.y, src),
+                            __shfl_sync(kFull, pk.cq.z, src), __shfl_sync(kFull, pk.cq.w, src));
+        if constexpr (kDipole) X[3] = __shfl_sync(kFull, pk.X3, src);
         const long long pid = __shfl_sync(kFull, pk.pid, src);
         const unsigned nsca = __shfl_sync(kFull, pk.n_sca, src);
-        const int tb = __shfl_sync(kFull, bin, src);
+        const int tb = kTable ? __shfl_sync(kFull, bin, src) : 0;
         const int t = __shfl_sync(kFull, t_next, src) + lane % per;
         // the packet's job (batched launches)
         Packet<T> jp;
@@ -1060,14 +1005,19 @@ __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Sme
                 __shfl_sync(kFull, reinterpret_cast<unsigned long long>(pk.job), src));
         bool acc = false;
         V3<T> n2{T(0), T(0), T(1)};
-        T mu = T(1);
+        T mu = T(1), Y[4];
         if (k < nu && t < P.max_trials) {
             const JobRef<T, B> job = job_of<T, B>(P, sm, jp);
             V3<T> th, ph;
-            stokes_basis(n, th, ph);
+            stokes_basis<kTable ? kFirst : kSecond>(n, th, ph);
             const Draw4<T> ut = draw4<T>(pid, nsca, 1u + (unsigned)t, P.seed, job.stream());
             T Pm[6];
-            acc = table_trial(job.t(), tb, ut, n, th, ph, X, n2, mu, Pm);
+            if constexpr (kTable)
+                acc = table_trial(job.t(), tb, ut, n, th, ph, X, n2, mu, Pm);
+            else if constexpr (kDipole)
+                acc = dipole_trial(dipole_const<T>(job.t().dip), q, ut, th, ph, X, n2, Y);
+            else
+                acc = rayleigh_trial(q, ut, n, th, ph, X, n2);
         }
         const unsigned am = __ballot_sync(kFull, acc);
         // each owner: the first accepted trial among its lanes
@@ -1076,16 +1026,20 @@ __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Sme
         const unsigned seg = own ? (per >= 32 ? kFull : ((1u << per) - 1u) << (kr * per)) : 0u;
         const unsigned hit = am & seg;
         const int w = hit != 0u ? __ffs(hit) - 1 : lane;
-        n2.x = __shfl_sync(kFull, n2.x, w);
-        n2.y = __shfl_sync(kFull, n2.y, w);
-        n2.z = __shfl_sync(kFull, n2.z, w);
-        mu = __shfl_sync(kFull, mu, w);
+        n2 = shfl3(n2, w);
+        if constexpr (kTable) mu = __shfl_sync(kFull, mu, w);
+        if constexpr (kDipole)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) Y[e] = __shfl_sync(kFull, Y[e], w);
         if (own) {
             if (hit != 0u) {
                 pk.trials += (unsigned)(w - kr * per + 1);
                 accepted = true;
                 n2a = n2;
-                mua = mu;
+                if constexpr (kTable) mua = mu;
+                if constexpr (kDipole)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) Ya[e] = Y[e];
             } else {
                 const int left = P.max_trials - t_next;
                 pk.trials += (unsigned)(left < per ? (left > 0 ? left : 0) : per);
@@ -1102,20 +1056,38 @@ __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Sme
     }
     const TablesDev& tabs = job_of<T, B>(P, sm, pk).t();
     const V3<T> n{pk.nx, pk.ny, pk.nz};
-    V3<T> th, ph, th2, ph2;
+    V3<T> th, ph;
     stokes_basis<kSecond>(n, th, ph);
-    stokes_basis(n2a, th2, ph2);
-    T Pm[6];
-    table_matrix(tabs.bins + (size_t)bin * tabs.n_theta * 2, tabs.n_theta, mua, Pm);
-    const PlaneRot<T> pr = plane_rotation<kFirst, kSecond, kSecond>(n, th, ph, n2a, th2, ph2);
-    const T X[4] = {pk.X0, pk.X1, pk.X2, pk.X3};
-    T Y[4];
-    apply_plane(pr, Pm, X, Y);
-    const T norm = X[0] / Y[0];
-    pk.X0 = Y[0] * norm;
-    pk.X1 = Y[1] * norm;
-    pk.X2 = Y[2] * norm;
-    pk.X3 = Y[3] * norm;
+    T norm;
+    if constexpr (kDipole) {
+        // the new Stokes vector is Zhat X (K_sca X)_0 / (s11 (Zhat X)_0), i.e. Zhat X renormalised
+        // to I + (s12 / s11) Q with Q in the grain-meridian basis
+        const DipoleConst<T> dp = dipole_const<T>(tabs.dip);
+        const GrainFrame<T> f = grain_frame(pk.cq, n, ph);
+        T Qg = pk.X1, Ug = pk.X2;
+        rotate_qu(Qg, Ug, f.c2, f.s2);
+        T S2 = (T(1) - f.cos_tp) * (T(1) + f.cos_tp);
+        S2 = S2 > T(0) ? S2 : T(0);
+        const T hs = (dp.cs1 - dp.cs0) * T(0.5) * S2;
+        const T Iw = pk.X0 + t_div(hs, dp.cs0 + hs) * Qg;
+        norm = Iw / Ya[0];
+    } else {
+        V3<T> th2, ph2;
+        stokes_basis(n2a, th2, ph2);
+        T Pm[6];
+        if constexpr (kTable)
+            table_matrix(tabs.bins + (size_t)bin * tabs.n_theta * 2, tabs.n_theta, mua, Pm);
+        else
+            rayleigh_matrix(dot(n, n2a), Pm);
+        const PlaneRot<T> pr = plane_rotation<kFirst, kTable ? kSecond : kFirst, kSecond>(n, th, ph, n2a, th2, ph2);
+        const T X[4] = {pk.X0, pk.X1, pk.X2, pk.X3};
+        apply_plane<kFirst, kTable ? kFirst : kSecond>(pr, Pm, X, Ya);
+        norm = X[0] / Ya[0];
+    }
+    pk.X0 = Ya[0] * norm;
+    pk.X1 = Ya[1] * norm;
+    pk.X2 = Ya[2] * norm;
+    pk.X3 = Ya[3] * norm;
     pk.nx = n2a.x;
     pk.ny = n2a.y;
     pk.nz = n2a.z;
@@ -1268,16 +1240,10 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
             if (__all_sync(kFull, pool_done)) break;
             continue;
         }
-        // scatterings of the warp run together once enough lanes wait for one
-        if (pend != 0u && (__popc(pend) >= scatter_batch<B, SCAT>() || work == 0u)) {
-            if constexpr (table_optics(SCAT)) {
-                scatter_coop<T, B>(P, sm, pk, alive, bt);  // every lane runs trials of the waiting packets
-            } else if constexpr (SCAT != kScatSurrogate) {  // the surrogate scatters in its own kernel
-                if (alive && pk.pending) {
-                    pk.pending = false;
-                    scatter_event<T, SCAT, B>(P, sm, pk, alive, bt);
-                }
-            }
+        // scatterings of the warp run together once enough lanes wait for one, or as many as move
+        if (pend != 0u && (__popc(pend) >= scatter_batch<B, SCAT>() || __popc(pend) >= __popc(work))) {
+            // every lane runs trials of the waiting packets (the surrogate scatters in its own kernel)
+            if constexpr (SCAT != kScatSurrogate) scatter_coop<T, SCAT, B>(P, sm, pk, alive, bt);
             continue;
         }
         int staged = 0;
