@@ -14,11 +14,81 @@ namespace mcrt {
 
 namespace {
 
-template <typename T> __global__ void __launch_bounds__(128) k_image(const __grid_constant__ ImageParams P) {
+// A ray's passage through one cell: the coefficients of its step in the grain-meridian
+// basis and the rotation into it.
+template <typename T> struct RayCell {
+    CellStep<T> k;
+    T c2, s2;
+};
+
+// Cell c of a ray of camera P.cam over the length ell: false when the cell leaves the ray as
+// it is.  The cell's record, grain frame and source are loaded together.
+template <typename T>
+__device__ __forceinline__ bool ray_cell(const ImageParams& P, const V3<T>& Om, const V3<T>& phc, long long c, T ell,
+                                         T inv_vol, RayCell<T>& o) {
+    const float4 r = __ldg(&P.g.cells[2 * c + 1]);
+    float4 q = make_float4(1.f, 0.f, 0.f, 0.f);
+    if (P.t.model == MCRT_SCAT_DIPOLE || !P.t.k_iso) q = __ldg(&P.g.cells[2 * c]);
+    double2 sa = make_double2(0.0, 0.0), sb = sa;
+    if (P.S) {
+        const double2* Sc = reinterpret_cast<const double2*>(P.S + ((size_t)c * P.n_cam + P.cam_index) * 4);
+        sa = __ldg(Sc);
+        sb = __ldg(Sc + 1);
+    }
+    const T ks = T(r.y);
+    const T kext = T(r.x) + ks;
+    if (!(kext > T(0) && ell > T(0))) return false;
+    const T omega = ks / kext;
+    T c2 = T(1), s2 = T(0), a1, a2, a3;
+    T s11 = omega, s12 = T(0);  // scattering part of K's first row
+    if (P.t.model == MCRT_SCAT_DIPOLE) {
+        const GrainFrame<T> f = grain_frame(q, Om, phc);
+        c2 = f.c2;
+        s2 = f.s2;
+        const DipoleConst<T> dp = dipole_const<T>(P.t.dip);
+        dipole_K(dp.ca0, dp.ca1, dp.cs0, dp.cs1, T(r.x) / kext, omega, f.cos_tp, a1, a2, s11, s12);
+        a3 = T(0);
+    } else if (P.t.k_iso) {
+        a1 = T(P.t.kext[0].x);
+        a2 = T(0);
+        a3 = T(0);
+    } else {
+        const GrainFrame<T> f = grain_frame<kSecond>(q, Om, phc);
+        c2 = f.c2;
+        s2 = f.s2;
+        kext_eval(P.t, P.t.kext, f.cos_tp, a1, a2, a3);
+    }
+    const T B = T(r.z);
+    // emission: the absorption part of K acting on (B, 0, 0, 0)
+    T S[4] = {(a1 - s11) * B, (a2 - s12) * B, T(0), T(0)};
+    if (P.S && ks > T(0)) {
+        const T f = omega * inv_vol;
+        T s1 = f * T(sa.y), s2v = f * T(sb.x);
+        rotate_qu(s1, s2v, c2, s2);
+        S[0] = t_fma(f, T(sa.x), S[0]);
+        S[1] += s1;
+        S[2] += s2v;
+        S[3] = t_fma(f, T(sb.y), S[3]);
+    }
+    o.k = cell_coeffs(a1, a2, a3, S, kext * ell);
+    o.c2 = c2;
+    o.s2 = s2;
+    return true;
+}
+
+// One ray per G lanes of a warp.  A ray is a serial chain, but only its walk (positions and
+// lengths) and the four-term step X <- e^{-K dtau} X + W are: the coefficients of a cell, some 400
+// instructions and the loads before them, do not depend on X.  All G lanes walk the next
+// G cells, lane j works out cell j, and the Stokes vector then passes through the cells in
+// order, so the result is that of one lane alone, bit for bit (R: grids with patches).
+template <typename T, int G, bool R>
+__global__ void __launch_bounds__(128) k_image(const __grid_constant__ ImageParams P) {
+    constexpr unsigned kAll = 0xffffffffu;
     const int nx = P.npix[0], ny = P.npix[1];
-    const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pix >= (long long)nx * ny) return;
-    const int ix = (int)(pix % nx), iy = (int)(pix / nx);
+    const long long pix = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    const int lane = threadIdx.x & 31, j_me = lane % G, first = lane - j_me;
+    const bool inside = pix < (long long)nx * ny;
+    const int ix = inside ? (int)(pix % nx) : 0, iy = inside ? (int)(pix / nx) : 0;
     GridT<T> g;
     for (int a = 0; a < 3; ++a) {
         g.n[a] = P.g.n[a];
@@ -50,92 +120,62 @@ template <typename T> __global__ void __launch_bounds__(128) k_image(const __gri
             miss = true;
         }
     }
-    T X[4] = {T(0), T(0), T(0), T(0)};
-    if (!miss && tin < tout) {
-        T p[3];
-        int idx[3];
-        for (int d = 0; d < 3; ++d) p[d] = o[d] + tin * dir[d];
-        for (int d = 0; d < 3; ++d) {
-            const T x = (p[d] - g.lo[d]) / g.d[d];
-            int i = (int)floor(x);
-            if (T(i) == x && dir[d] < T(0)) i -= 1;
-            i = i < 0 ? 0 : (i >= g.n[d] ? g.n[d] - 1 : i);
-            idx[d] = i;
+    bool on = inside && !miss && tin < tout;  // the ray has cells left
+    T p[3];
+    int idx[3];
+    for (int d = 0; d < 3; ++d) p[d] = on ? o[d] + tin * dir[d] : g.lo[d];
+    for (int d = 0; d < 3; ++d) {
+        const T x = (p[d] - g.lo[d]) / g.d[d];
+        int i = (int)floor(x);
+        if (T(i) == x && dir[d] < T(0)) i -= 1;
+        i = i < 0 ? 0 : (i >= g.n[d] ? g.n[d] - 1 : i);
+        idx[d] = i;
+    }
+    const T inv_vol_root = T(1.0 / (P.g.d[0] * P.g.d[1] * P.g.d[2]));
+    T inv_vol = inv_vol_root;
+    // composite grid: the current level's geometry (root, or the patch the ray is in)
+    GridT<T> gc = g;
+    int lvl = 0;
+    auto descend = [&]() {
+        const long long rc = ((long long)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
+        const int q = covering_patch(P.g.cells[2 * rc + 1]);
+        if (q < 0) return;
+        const PatchDev& pq = P.g.patches[q];
+        lvl = q + 1;
+        for (int a = 0; a < 3; ++a) {
+            gc.n[a] = pq.n[a];
+            gc.lo[a] = patch_lo<T>(pq, a);
+            gc.d[a] = patch_d<T>(pq, a);
         }
-        const T inv_vol_root = T(1.0 / (P.g.d[0] * P.g.d[1] * P.g.d[2]));
-        T inv_vol = inv_vol_root;
-        // composite grid: the current level's geometry (root, or the patch the ray is in)
-        GridT<T> gc = g;
-        int lvl = 0;
-        auto descend = [&]() {
-            const long long rc = ((long long)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0];
-            const int q = covering_patch(P.g.cells[2 * rc + 1]);
-            if (q < 0) return;
-            const PatchDev& pq = P.g.patches[q];
-            lvl = q + 1;
-            for (int a = 0; a < 3; ++a) {
-                gc.n[a] = pq.n[a];
-                gc.lo[a] = patch_lo<T>(pq, a);
-                gc.d[a] = patch_d<T>(pq, a);
-            }
-            inv_vol = T(1.0 / (pq.d[0] * pq.d[1] * pq.d[2]));
-            patch_locate<T>(pq, p[0], p[1], p[2], dir[0], dir[1], dir[2], idx);
-        };
-        if (P.g.n_patches > 0) descend();
-        const long long max_steps =
-            (long long)(g.n[0] + g.n[1] + g.n[2]) * (P.g.n_patches > 0 ? 3 * 16 + 1 : 1) + 3;
-        for (long long step = 0; step < max_steps; ++step) {
+        inv_vol = T(1.0 / (pq.d[0] * pq.d[1] * pq.d[2]));
+        patch_locate<T>(pq, p[0], p[1], p[2], dir[0], dir[1], dir[2], idx);
+    };
+    if constexpr (R)
+        if (on) descend();
+    long long left = (long long)(g.n[0] + g.n[1] + g.n[2]) * (R ? 3 * 16 + 1 : 1) + 3;  // bound on the cells
+    T X[4] = {T(0), T(0), T(0), T(0)};
+    while (__any_sync(kAll, on)) {
+        T my_ell = T(0), my_vol = inv_vol_root;
+        long long my_c = -1;
+#pragma unroll 1
+        for (int j = 0; j < G; ++j) {
+            if (!on) continue;
             int axis;
             const T ell = exit_distance(gc, idx, p, dir, axis);
-            if (axis < 0) break;
-            const long long c = lvl == 0 ? ((long long)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0]
-                                         : patch_cell(P.g.patches[lvl - 1], idx[0], idx[1], idx[2]);
-            const float4 r = P.g.cells[2 * c + 1];
-            const T ks = T(r.y);
-            const T kext = T(r.x) + ks;
-            if (kext > T(0) && ell > T(0)) {
-                const T omega = ks / kext;
-                T c2 = T(1), s2 = T(0), a1, a2, a3;
-                T s11 = omega, s12 = T(0);  // scattering part of K's first row
-                if (P.t.model == MCRT_SCAT_DIPOLE) {
-                    const GrainFrame<T> f = grain_frame(P.g.cells[2 * c], Om, phc);
-                    c2 = f.c2;
-                    s2 = f.s2;
-                    const DipoleConst<T> dp = dipole_const<T>(P.t.dip);
-                    dipole_K(dp.ca0, dp.ca1, dp.cs0, dp.cs1, T(r.x) / kext, omega, f.cos_tp, a1,
-                             a2, s11, s12);
-                    a3 = T(0);
-                } else if (P.t.k_iso) {
-                    a1 = T(P.t.kext[0].x);
-                    a2 = T(0);
-                    a3 = T(0);
-                } else {
-                    const float4 q = P.g.cells[2 * c];
-                    const GrainFrame<T> f = grain_frame<kSecond>(q, Om, phc);
-                    c2 = f.c2;
-                    s2 = f.s2;
-                    kext_eval(P.t, P.t.kext, f.cos_tp, a1, a2, a3);
-                }
-                const T B = T(r.z);
-                // emission: the absorption part of K acting on (B, 0, 0, 0)
-                T S[4] = {(a1 - s11) * B, (a2 - s12) * B, T(0), T(0)};
-                if (P.S && ks > T(0)) {
-                    const double* Sc = P.S + ((size_t)c * P.n_cam + P.cam_index) * 4;
-                    const T f = omega * inv_vol;
-                    T s1 = f * T(Sc[1]), s2v = f * T(Sc[2]);
-                    rotate_qu(s1, s2v, c2, s2);
-                    S[0] += f * T(Sc[0]);
-                    S[1] += s1;
-                    S[2] += s2v;
-                    S[3] += f * T(Sc[3]);
-                }
-                rotate_qu(X[1], X[2], c2, s2);
-                cell_step(cell_coeffs(a1, a2, a3, S, kext * ell), X);
-                rotate_back(X[1], X[2], c2, s2);
+            if (axis < 0 || left-- <= 0) {
+                on = false;
+                continue;
             }
-            if (lvl == 0) {
-                if (!cross_face(g, idx, p, dir, ell, axis)) break;
-                if (P.g.n_patches > 0) descend();
+            if (j == j_me) {
+                my_ell = ell;
+                my_vol = inv_vol;
+                my_c = !R || lvl == 0 ? ((long long)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0]
+                                      : patch_cell(P.g.patches[lvl - 1], idx[0], idx[1], idx[2]);
+            }
+            if (!R || lvl == 0) {
+                on = cross_face(g, idx, p, dir, ell, axis);
+                if constexpr (R)
+                    if (on) descend();
             } else if (!cross_face(gc, idx, p, dir, ell, axis)) {
                 // out of the patch: the root cell beyond its face
                 const PatchDev& pq = P.g.patches[lvl - 1];
@@ -144,12 +184,32 @@ template <typename T> __global__ void __launch_bounds__(128) k_image(const __gri
                 lvl = 0;
                 gc = g;
                 inv_vol = inv_vol_root;
-                if (idx[axis] < 0 || idx[axis] >= g.n[axis]) break;
-                descend();
+                on = idx[axis] >= 0 && idx[axis] < g.n[axis];
+                if (on) descend();
+            }
+        }
+        RayCell<T> rc;
+        const bool act = my_c >= 0 && ray_cell(P, Om, phc, my_c, my_ell, my_vol, rc);
+        const unsigned any = __ballot_sync(kAll, act);
+#pragma unroll 1
+        for (int j = 0; j < G; ++j) {
+            if (act && j == j_me) {
+                rotate_qu(X[1], X[2], rc.c2, rc.s2);
+                cell_step(rc.k, X);
+                rotate_back(X[1], X[2], rc.c2, rc.s2);
+            }
+            if constexpr (G > 1) {
+                static_assert(G == 4 || G == 8);
+                constexpr unsigned kGroups = G == 8 ? 0x01010101u : 0x11111111u;  // lane 0 of each ray
+                if (any & (kGroups << j)) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) X[e] = __shfl_sync(kAll, X[e], first + j);
+                }
             }
         }
     }
-    for (int e = 0; e < 4; ++e) P.out[((size_t)e * ny + iy) * nx + ix] = (double)X[e];
+    if (inside && j_me == 0)
+        for (int e = 0; e < 4; ++e) P.out[((size_t)e * ny + iy) * nx + ix] = (double)X[e];
 }
 
 // ---------------------------------------------------------------------------------
@@ -522,15 +582,39 @@ cudaError_t launch_dipole_setup(double eps_re, double eps_im, double aspect, dou
     return cudaGetLastError();
 }
 
+template <typename T, int G> static void image_launch(const ImageParams& p, int block, cudaStream_t s) {
+    const long long threads = (long long)p.npix[0] * p.npix[1] * G;
+    const unsigned grid = (unsigned)((threads + block - 1) / block);
+    if (p.g.n_patches > 0)
+        k_image<T, G, true><<<grid, block, 0, s>>>(p);
+    else
+        k_image<T, G, false><<<grid, block, 0, s>>>(p);
+}
+
+// Lanes per ray: the fewer rays, the more of a ray's cells are worked out at once; with enough
+// rays to fill the SMs the shared walk only repeats work.  Measured per image, us with 8, 4 and 1
+// lanes (and one ray per lane before): FP32, 96^3 disk, 64^2 81, 101, 256 (271); 128^2 125, 122,
+// 245 (301); 181^2 204, 150, 238 (286); 256^2 361, 246, 247 (293); FP64, 24^3 disk, 32^2 96, 135,
+// 325 (326); 64^2 174, 131, 326 (327); 128^2 590, 408, 319 (320).  Blocks of 64 keep FP64's last
+// wave short (256^2: 801 us against 856 with 128); pixel tiles of 8 x 4 per warp gave FP32 no more
+// than 2 % at 512^2 and lost 6 % at 256^2 against rows.
+template <typename T> static void image_launch(const ImageParams& p, cudaStream_t s) {
+    constexpr long long kRays8 = sizeof(T) == 4 ? 12288 : 2048, kRays4 = sizeof(T) == 4 ? 40960 : 8192;
+    const long long rays = (long long)p.npix[0] * p.npix[1];
+    if (rays <= kRays8)
+        image_launch<T, 8>(p, 64, s);
+    else if (rays <= kRays4)
+        image_launch<T, 4>(p, 128, s);
+    else
+        image_launch<T, 1>(p, sizeof(T) == 4 ? 128 : 64, s);
+}
+
 cudaError_t launch_image(const ImageParams& p, int precision, cudaStream_t s) {
-    const long long npix = (long long)p.npix[0] * p.npix[1];
-    const int block = 128;
-    const unsigned grid = (unsigned)((npix + block - 1) / block);
     (void)cudaGetLastError();  // report this launch's error only
     if (precision == MCRT_FP64)
-        k_image<double><<<grid, block, 0, s>>>(p);
+        image_launch<double>(p, s);
     else
-        k_image<float><<<grid, block, 0, s>>>(p);
+        image_launch<float>(p, s);
     return cudaGetLastError();
 }
 
