@@ -252,6 +252,8 @@ __global__ void k_setup_cells(const float* __restrict__ ka, const float* __restr
     }
 }
 
+constexpr int kPrepBlock = 256, kMaxAngles = 721, kMaxBins = 32;  // limits of mcrt_set_dust_tables
+
 // Table preparation (one block): mixture matrix for the tally, per-bin rows,
 // piecewise-constant envelope of P11 with its normalised cumulative weights,
 // cumulative bin weights, extinction rows and the sphere average of alpha1.  The two
@@ -259,66 +261,104 @@ __global__ void k_setup_cells(const float* __restrict__ ka, const float* __restr
 // doubles and as many floats, bin_cdf n_bins doubles and n_bins floats), as are the cosines of
 // the tabulated angles (n_theta doubles, n_theta floats, each the limit of an interval as a
 // trial in that precision would compute it).
-__global__ void k_prepare_tables(int model, int n_bins, int n_theta, int n_ktheta, const float* __restrict__ mueller,
-                                 const float* __restrict__ bin_weight, const float* __restrict__ kext,
-                                 float4* __restrict__ mix, float4* __restrict__ bins, double* __restrict__ env_cdf,
-                                 float* __restrict__ env, double* __restrict__ bin_cdf, double* __restrict__ cosines,
-                                 float4* __restrict__ kext4, double* __restrict__ alpha1_mean) {
+// The FP64 trigonometry is the cost: every angle is evaluated once, spread over the block, and
+// only the additions of the cumulative sums stay serial (one lane per bin, one lane for alpha1),
+// in the order of the angles.  8 bins of 181 angles: 43 us; 1081 us with one thread per bin
+// evaluating two cosines for each of its intervals (32 bins of 721: 240 and 4604).
+__global__ void __launch_bounds__(kPrepBlock)
+    k_prepare_tables(int model, int n_bins, int n_theta, int n_ktheta, const float* __restrict__ mueller,
+                     const float* __restrict__ bin_weight, const float* __restrict__ kext, float4* __restrict__ mix,
+                     float4* __restrict__ bins, double* __restrict__ env_cdf, float* __restrict__ env,
+                     double* __restrict__ bin_cdf, double* __restrict__ cosines, float4* __restrict__ kext4,
+                     double* __restrict__ alpha1_mean) {
     const double pi = 3.141592653589793;
-    for (int j = threadIdx.x; j < n_ktheta; j += blockDim.x)
+    const bool table = model == MCRT_SCAT_TABLE;
+    const int nint = n_theta - 1;
+    __shared__ double ck[kMaxAngles], sk[kMaxAngles], ca[kMaxAngles];  // of the extinction's and the matrix's angles
+    __shared__ double share[kMaxBins], total[kMaxBins];
+    const double h = pi / (n_ktheta - 1);
+    for (int j = threadIdx.x; j < n_ktheta; j += blockDim.x) {
         kext4[j] = make_float4(kext[3 * j], kext[3 * j + 1], kext[3 * j + 2], 0.f);
-    if (threadIdx.x == 0) {
-        const double h = pi / (n_ktheta - 1);
-        double s = 0.0;
-        for (int j = 0; j + 1 < n_ktheta; ++j) {
-            const double ta = j * h, tb = (j + 1) * h;
-            const double A = kext[3 * j], B = ((double)kext[3 * (j + 1)] - A) / h;
-            s += A * (cos(ta) - cos(tb)) + B * (-(tb - ta) * cos(tb) + sin(tb) - sin(ta));
-        }
-        *alpha1_mean = 0.5 * s;
+        ck[j] = cos(j * h);
+        sk[j] = sin(j * h);
     }
-    if (model != MCRT_SCAT_TABLE) return;
-    __shared__ double wsum_s;
-    if (threadIdx.x == 0) {
+    if (table)
+        for (int j = threadIdx.x; j < n_theta; j += blockDim.x) ca[j] = cos(pi * j / nint);
+    if (table && threadIdx.x == 0) {
         double ws = 0.0;
         for (int k = 0; k < n_bins; ++k) ws += bin_weight[k];
         double acc = 0.0;
         for (int k = 0; k < n_bins; ++k) {
             acc += bin_weight[k];
             bin_cdf[k] = acc / ws;
+            share[k] = (double)bin_weight[k] / ws;
         }
-        wsum_s = ws;
     }
     __syncthreads();
-    const double ws = wsum_s;
-    for (int j = threadIdx.x; j < n_theta; j += blockDim.x) {
-        double m[6] = {0, 0, 0, 0, 0, 0};
-        for (int k = 0; k < n_bins; ++k) {
-            const float* row = mueller + ((size_t)k * n_theta + j) * 6;
-            bins[((size_t)k * n_theta + j) * 2] = make_float4(row[0], row[1], row[2], row[3]);
-            bins[((size_t)k * n_theta + j) * 2 + 1] = make_float4(row[4], row[5], 0.f, 0.f);
-            for (int e = 0; e < 6; ++e) m[e] += (double)bin_weight[k] / ws * row[e];
+    // the terms of alpha1's average and the steps of the cumulative weights, in place
+    double term[kMaxAngles / kPrepBlock + 1], step[kMaxAngles / kPrepBlock + 1];
+#pragma unroll
+    for (int i = 0; i <= kMaxAngles / kPrepBlock; ++i) {
+        const int j = threadIdx.x + i * kPrepBlock;
+        if (j + 1 < n_ktheta) {
+            const double width = __dsub_rn(__dmul_rn(j + 1, h), __dmul_rn(j, h));
+            const double A = kext[3 * j], B = ((double)kext[3 * (j + 1)] - A) / h;
+            const double q = __dsub_rn(fma(-width, ck[j + 1], sk[j + 1]), sk[j]);
+            term[i] = fma(B, q, __dmul_rn(A, ck[j] - ck[j + 1]));
         }
-        mix[2 * j] = make_float4((float)m[0], (float)m[1], (float)m[2], (float)m[3]);
-        mix[2 * j + 1] = make_float4((float)m[4], (float)m[5], 0.f, 0.f);
+        if (table && j < nint) step[i] = ca[j] - ca[j + 1];
     }
-    const int nint = n_theta - 1;
-    for (int k = threadIdx.x; k < n_bins; k += blockDim.x) {
-        const float* tab = mueller + (size_t)k * n_theta * 6;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i <= kMaxAngles / kPrepBlock; ++i) {
+        const int j = threadIdx.x + i * kPrepBlock;
+        if (j + 1 < n_ktheta) ck[j] = term[i];
+        if (table && j < nint) ca[j] = step[i];
+    }
+    __syncthreads();
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    if (warp == 0 && lane == 0) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int j = 0; j + 1 < n_ktheta; ++j) s += ck[j];
+        *alpha1_mean = 0.5 * s;
+    }
+    if (!table) return;
+    if (warp == 1 && lane < n_bins) {
+        const float* tab = mueller + (size_t)lane * n_theta * 6;
         double tot = 0.0;
+        float ea = tab[0];
+#pragma unroll 8
         for (int j = 0; j < nint; ++j) {
-            const double e = fmax((double)tab[j * 6], (double)tab[(j + 1) * 6]);
-            tot += e * (cos(pi * j / nint) - cos(pi * (j + 1) / nint));
-            env[(size_t)k * nint + j] = (float)e;
-            env_cdf[(size_t)k * nint + j] = tot;
+            const float eb = tab[(j + 1) * 6];
+            const double e = fmax((double)ea, (double)eb);
+            tot = fma(e, ca[j], tot);
+            env[(size_t)lane * nint + j] = (float)e;
+            env_cdf[(size_t)lane * nint + j] = tot;
+            ea = eb;
         }
-        for (int j = 0; j < nint; ++j) env_cdf[(size_t)k * nint + j] /= tot;
+        total[lane] = tot;
+    } else if (warp > 1) {
+        for (int j = threadIdx.x - 64; j < n_theta; j += blockDim.x - 64) {
+            double m[6] = {0, 0, 0, 0, 0, 0};
+            for (int k = 0; k < n_bins; ++k) {
+                const float* row = mueller + ((size_t)k * n_theta + j) * 6;
+                bins[((size_t)k * n_theta + j) * 2] = make_float4(row[0], row[1], row[2], row[3]);
+                bins[((size_t)k * n_theta + j) * 2 + 1] = make_float4(row[4], row[5], 0.f, 0.f);
+                for (int e = 0; e < 6; ++e) m[e] = fma(share[k], (double)row[e], m[e]);
+            }
+            mix[2 * j] = make_float4((float)m[0], (float)m[1], (float)m[2], (float)m[3]);
+            mix[2 * j + 1] = make_float4((float)m[4], (float)m[5], 0.f, 0.f);
+        }
     }
-    // FP32 copies after the FP64 tables
     __syncthreads();
     float* env_cdf_f = reinterpret_cast<float*>(env_cdf + (size_t)n_bins * nint);
     float* bin_cdf_f = reinterpret_cast<float*>(bin_cdf + n_bins);
-    for (int i = threadIdx.x; i < n_bins * nint; i += blockDim.x) env_cdf_f[i] = (float)env_cdf[i];
+    for (int i = threadIdx.x; i < n_bins * nint; i += blockDim.x) {
+        const double v = env_cdf[i] / total[i / nint];
+        env_cdf[i] = v;
+        env_cdf_f[i] = (float)v;
+    }
     for (int k = threadIdx.x; k < n_bins; k += blockDim.x) bin_cdf_f[k] = (float)bin_cdf[k];
     float* cos_f = reinterpret_cast<float*>(cosines + n_theta);
     for (int j = threadIdx.x; j < n_theta; j += blockDim.x) {
@@ -635,7 +675,7 @@ cudaError_t launch_prepare_tables(int model, int n_bins, int n_theta, int n_kthe
                                   double* env_cdf, float* env, double* bin_cdf, double* cosines, float4* kext4,
                                   double* alpha1_mean, cudaStream_t s) {
     (void)cudaGetLastError();  // report this launch's error only
-    k_prepare_tables<<<1, 256, 0, s>>>(model, n_bins, n_theta, n_ktheta, mueller, bin_weight, kext, mix, bins,
+    k_prepare_tables<<<1, kPrepBlock, 0, s>>>(model, n_bins, n_theta, n_ktheta, mueller, bin_weight, kext, mix, bins,
                                        env_cdf, env, bin_cdf, cosines, kext4, alpha1_mean);
     return cudaGetLastError();
 }
