@@ -23,16 +23,16 @@ struct mcrt_ctx {
     cudaStream_t stream = nullptr;
     int device = 0;
     int n_sm = 0;
-    float4* d_cells = nullptr;
+    float4* d_cells = nullptr;      // one allocation: cells, work area, patches
     PatchDev* d_patches = nullptr;  // static mesh refinement
     bool has_emissivity = false;
-    // optics
+    // optics: one allocation, that of d_kext
     bool tables_set = false;
     TablesDev t{};
     float4 *d_mix = nullptr, *d_bins = nullptr, *d_kext = nullptr;
     double *d_env_cdf = nullptr, *d_bin_cdf = nullptr, *d_cos = nullptr, *d_alpha1 = nullptr;
     float* d_env = nullptr;
-    // thermal emission CDF
+    // thermal emission CDF: one allocation, that of d_cdf
     double* d_cdf = nullptr;
     double* d_block_sums = nullptr;
     long long* d_guide = nullptr;
@@ -62,7 +62,7 @@ struct mcrt_ctx {
     float4* d_records = nullptr;
     unsigned long long rec_cap = 0;
     size_t rec_bytes = 0;  // size of the tally-record queue allocation
-    float4 *d_susp = nullptr, *d_res = nullptr;
+    float4 *d_susp = nullptr, *d_res = nullptr;  // one allocation
     unsigned long long wave_cap = 0;
     // work area: counter (8 B), stats (16 x 8 B), status (8 B)
     unsigned char* d_work = nullptr;
@@ -102,26 +102,44 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Device copy of a caller buffer: the buffer itself if it is device memory, else
-// a temporary allocation filled from host memory.
+// Device copies of a caller's buffers: a buffer itself if it is device memory, else its
+// part of one temporary allocation, filled from host memory.  An allocation and its free
+// cost 60 us and more whatever their size, as much as a small model's set-up kernels, so
+// what lives together is allocated together here and below.
 struct DevIn {
-    const void* ptr = nullptr;
     void* owned = nullptr;
     ~DevIn() {
         if (owned) cudaFree(owned);
     }
 };
 
-cudaError_t stage(DevIn& d, const void* src, size_t bytes, cudaStream_t s) {
-    if (!src) return cudaSuccess;
-    if (is_device_ptr(src)) {
-        d.ptr = src;
-        return cudaSuccess;
+struct Buffer {
+    const void* src;
+    size_t bytes;
+    const void* ptr;  // on the device, after stage()
+};
+
+constexpr size_t round256(size_t n) { return (n + 255) & ~(size_t)255; }
+
+cudaError_t stage(DevIn& d, Buffer* in, int n, cudaStream_t s) {
+    size_t total = 0;
+    for (int i = 0; i < n; ++i) {
+        in[i].ptr = in[i].src;
+        if (in[i].src && !is_device_ptr(in[i].src)) {
+            in[i].ptr = nullptr;
+            total += round256(in[i].bytes);
+        }
     }
-    cudaError_t e = cudaMalloc(&d.owned, bytes);
-    if (e != cudaSuccess) return e;
-    d.ptr = d.owned;
-    return cudaMemcpyAsync(d.owned, src, bytes, cudaMemcpyHostToDevice, s);
+    if (total == 0) return cudaSuccess;
+    cudaError_t e = cudaMalloc(&d.owned, total);
+    unsigned char* at = static_cast<unsigned char*>(d.owned);
+    for (int i = 0; i < n && e == cudaSuccess; ++i)
+        if (in[i].src && !in[i].ptr) {
+            in[i].ptr = at;
+            e = cudaMemcpyAsync(at, in[i].src, in[i].bytes, cudaMemcpyHostToDevice, s);
+            at += round256(in[i].bytes);
+        }
+    return e;
 }
 
 // Stokes basis of a unit vector on the host (phi-hat = (-y, x, 0)/rho,
@@ -159,7 +177,6 @@ void free_wave(mcrt_ctx* c) {
     cudaFree(c->d_wave);
     cudaFree(c->d_records);
     cudaFree(c->d_susp);
-    cudaFree(c->d_res);
     c->d_wave = nullptr;
     c->d_records = nullptr;
     c->d_susp = c->d_res = nullptr;
@@ -169,14 +186,7 @@ void free_wave(mcrt_ctx* c) {
 
 void free_tables(mcrt_ctx* c) {
     free_surrogate(c);  // the network was attached for these tables
-    cudaFree(c->d_mix);
-    cudaFree(c->d_bins);
     cudaFree(c->d_kext);
-    cudaFree(c->d_env_cdf);
-    cudaFree(c->d_bin_cdf);
-    cudaFree(c->d_cos);
-    cudaFree(c->d_alpha1);
-    cudaFree(c->d_env);
     c->d_mix = c->d_bins = c->d_kext = nullptr;
     c->d_env_cdf = c->d_bin_cdf = c->d_cos = c->d_alpha1 = nullptr;
     c->d_env = nullptr;
@@ -272,9 +282,13 @@ static mcrt_status create_grid(const char* me, mcrt_ctx** out, int32_t nx, int32
     c->has_emissivity = emissivity != nullptr;
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_cells, (size_t)ncell * 2 * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_work, kWorkBytes);
-    if (e == cudaSuccess && n_patches > 0) e = cudaMalloc(&c->d_patches, hp.size() * sizeof(PatchDev));
+    const size_t cell_bytes = round256((size_t)ncell * 2 * sizeof(float4));
+    if (e == cudaSuccess)
+        e = cudaMalloc(&c->d_cells, cell_bytes + round256(kWorkBytes) + hp.size() * sizeof(PatchDev));
+    if (e == cudaSuccess) {
+        c->d_work = reinterpret_cast<unsigned char*>(c->d_cells) + cell_bytes;
+        if (n_patches > 0) c->d_patches = reinterpret_cast<PatchDev*>(c->d_work + round256(kWorkBytes));
+    }
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
     if (e != cudaSuccess) {
@@ -291,15 +305,13 @@ static mcrt_status create_grid(const char* me, mcrt_ctx** out, int32_t nx, int32
     // cell records of one level: its arrays staged on the device, then k_setup_cells
     auto level = [&](const float* ka_in, const float* ks_in, const float* bf_in, const float* em_in, long long count,
                      float4* dst) {
-        DevIn ka, ks, bf, em;
+        DevIn d;
         const size_t fb = (size_t)count * sizeof(float);
-        cudaError_t r = stage(ka, ka_in, fb, c->stream);
-        if (r == cudaSuccess) r = stage(ks, ks_in, fb, c->stream);
-        if (r == cudaSuccess) r = stage(bf, bf_in, 3 * fb, c->stream);
-        if (r == cudaSuccess) r = stage(em, em_in, fb, c->stream);
+        Buffer in[4] = {{ka_in, fb, nullptr}, {ks_in, fb, nullptr}, {bf_in, 3 * fb, nullptr}, {em_in, fb, nullptr}};
+        cudaError_t r = stage(d, in, 4, c->stream);
         if (r == cudaSuccess)
-            r = launch_setup_cells((const float*)ka.ptr, (const float*)ks.ptr, (const float*)bf.ptr,
-                                   (const float*)em.ptr, count, dst, (unsigned*)c->d_work, c->stream);
+            r = launch_setup_cells((const float*)in[0].ptr, (const float*)in[1].ptr, (const float*)in[2].ptr,
+                                   (const float*)in[3].ptr, count, dst, (unsigned*)c->d_work, c->stream);
         // the staged copies are freed when this returns: finish the kernel first
         if (r == cudaSuccess) r = cudaStreamSynchronize(c->stream);
         return r;
@@ -387,29 +399,44 @@ mcrt_status mcrt_set_dust_tables(mcrt_ctx* ctx, int32_t model, int32_t n_bins, i
     const int nint = n_theta > 1 ? n_theta - 1 : 1;
     const int nb = n_bins > 0 ? n_bins : 1;
     const int nt = n_theta > 0 ? n_theta : 1;
-    cudaError_t e = cudaMalloc(&ctx->d_kext, n_ktheta * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_alpha1, sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_mix, (size_t)nt * 2 * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_bins, (size_t)nb * nt * 2 * sizeof(float4));
-    // cumulative tables: FP64, then their FP32 copies
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_env_cdf, (size_t)nb * nint * (sizeof(double) + sizeof(float)));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_env, (size_t)nb * nint * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_bin_cdf, (size_t)nb * (sizeof(double) + sizeof(float)));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_cos, (size_t)nt * (sizeof(double) + sizeof(float)));
+    // cumulative tables and cosines: FP64, then their FP32 copies
+    const size_t both = sizeof(double) + sizeof(float);
+    size_t total = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = total;
+        total += round256(bytes);
+        return at;
+    };
+    const size_t at_kext = part((size_t)n_ktheta * sizeof(float4)), at_alpha1 = part(sizeof(double)),
+                 at_mix = part((size_t)nt * 2 * sizeof(float4)), at_bins = part((size_t)nb * nt * 2 * sizeof(float4)),
+                 at_env_cdf = part((size_t)nb * nint * both), at_env = part((size_t)nb * nint * sizeof(float)),
+                 at_bin_cdf = part((size_t)nb * both), at_cos = part((size_t)nt * both);
+    cudaError_t e = cudaMalloc(&ctx->d_kext, total);
+    if (e == cudaSuccess) {
+        unsigned char* const base = reinterpret_cast<unsigned char*>(ctx->d_kext) - at_kext;
+        ctx->d_alpha1 = reinterpret_cast<double*>(base + at_alpha1);
+        ctx->d_mix = reinterpret_cast<float4*>(base + at_mix);
+        ctx->d_bins = reinterpret_cast<float4*>(base + at_bins);
+        ctx->d_env_cdf = reinterpret_cast<double*>(base + at_env_cdf);
+        ctx->d_env = reinterpret_cast<float*>(base + at_env);
+        ctx->d_bin_cdf = reinterpret_cast<double*>(base + at_bin_cdf);
+        ctx->d_cos = reinterpret_cast<double*>(base + at_cos);
+    }
     if (e != cudaSuccess) {
         free_tables(ctx);
         return fail(ctx, MCRT_E_NOMEM, "mcrt_set_dust_tables: %s", cudaGetErrorString(e));
     }
     double a1m = 0.0;
     {
-        DevIn dm, dw, dk;
-        e = stage(dk, kext, (size_t)n_ktheta * 3 * sizeof(float), ctx->stream);
-        if (e == cudaSuccess && model == MCRT_SCAT_TABLE)
-            e = stage(dm, mueller, (size_t)n_bins * n_theta * 6 * sizeof(float), ctx->stream);
-        if (e == cudaSuccess && model == MCRT_SCAT_TABLE) e = stage(dw, bin_weight, (size_t)n_bins * sizeof(float), ctx->stream);
+        const bool table = model == MCRT_SCAT_TABLE;
+        DevIn d;
+        Buffer in[3] = {{kext, (size_t)n_ktheta * 3 * sizeof(float), nullptr},
+                        {table ? mueller : nullptr, (size_t)n_bins * n_theta * 6 * sizeof(float), nullptr},
+                        {table ? bin_weight : nullptr, (size_t)n_bins * sizeof(float), nullptr}};
+        e = stage(d, in, 3, ctx->stream);
         if (e == cudaSuccess)
-            e = launch_prepare_tables(model, n_bins, n_theta, n_ktheta, (const float*)dm.ptr, (const float*)dw.ptr,
-                                      (const float*)dk.ptr, ctx->d_mix, ctx->d_bins, ctx->d_env_cdf, ctx->d_env,
+            e = launch_prepare_tables(model, n_bins, n_theta, n_ktheta, (const float*)in[1].ptr, (const float*)in[2].ptr,
+                                      (const float*)in[0].ptr, ctx->d_mix, ctx->d_bins, ctx->d_env_cdf, ctx->d_env,
                                       ctx->d_bin_cdf, ctx->d_cos, ctx->d_kext, ctx->d_alpha1, ctx->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&a1m, ctx->d_alpha1, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -594,11 +621,16 @@ static mcrt_status prepare_model(mcrt_ctx* ctx, const mcrt_launch_desc* d, uint3
         return fail(ctx, MCRT_E_INVAL, "mcrt_launch_packets: thermal source needs an emissivity grid");
     if (need_thermal && !ctx->cdf_valid) {
         const int nb = thermal_cdf_blocks(ctx->g.ncell);
-        if (!ctx->d_cdf) CK(ctx, cudaMalloc(&ctx->d_cdf, (size_t)ctx->g.ncell * sizeof(double)));
-        if (!ctx->d_block_sums) CK(ctx, cudaMalloc(&ctx->d_block_sums, (size_t)nb * sizeof(double)));
-        CK(ctx, launch_thermal_cdf(ctx->g, ctx->t.alpha1_mean, ctx->d_cdf, ctx->d_block_sums, nb, ctx->stream));
         ctx->n_guide = ctx->g.ncell < (1ll << 22) ? ctx->g.ncell : (1ll << 22);
-        if (!ctx->d_guide) CK(ctx, cudaMalloc(&ctx->d_guide, (size_t)(ctx->n_guide + 1) * sizeof(long long)));
+        if (!ctx->d_cdf) {
+            const size_t at_sums = round256((size_t)ctx->g.ncell * sizeof(double));
+            const size_t at_guide = at_sums + round256((size_t)nb * sizeof(double));
+            CK(ctx, cudaMalloc(&ctx->d_cdf, at_guide + (size_t)(ctx->n_guide + 1) * sizeof(long long)));
+            unsigned char* const base = reinterpret_cast<unsigned char*>(ctx->d_cdf);
+            ctx->d_block_sums = reinterpret_cast<double*>(base + at_sums);
+            ctx->d_guide = reinterpret_cast<long long*>(base + at_guide);
+        }
+        CK(ctx, launch_thermal_cdf(ctx->g, ctx->t.alpha1_mean, ctx->d_cdf, ctx->d_block_sums, nb, ctx->stream));
         CK(ctx, launch_thermal_guide(ctx->d_cdf, ctx->g.ncell, ctx->d_guide, ctx->n_guide, ctx->stream));
         CK(ctx, cudaMemcpyAsync(&ctx->thermal_total, ctx->d_cdf + (ctx->g.ncell - 1), sizeof(double),
                                 cudaMemcpyDeviceToHost, ctx->stream));
@@ -783,24 +815,26 @@ static mcrt_status launch_one(mcrt_ctx* ctx, const mcrt_launch_desc* d, mcrt_sta
         const unsigned long long margin =
             (unsigned long long)ctx->n_sm * (16ull * 128ull + 64ull * 32ull * (unsigned long long)MCRT_REC_CHUNK);
         // queue: 32 records per packet in flight for the network's 64-byte records,
-        // MCRT_TABLE_ROUND_RECORDS for the tables' 32-byte records, two slots of them (the
-        // overlapped rounds fill one while the tally reads the other)
+        // MCRT_TABLE_ROUND_RECORDS for the tables' 32-byte records; overlapped rounds have two
+        // slots of them and fill one while the tally reads the other.
+        // Overlap of a round's tally with the next transport is opt-in: measured slower on the
+        // disk (the latency-bound transport slows down under the tally's DRAM traffic)
+        const bool overlap = !sur && d->tally_blocks_per_sm > 0;
         const unsigned long long per_packet = sur ? 32ull : (unsigned long long)MCRT_TABLE_ROUND_RECORDS;
-        const size_t rec_bytes = (size_t)(sur ? kRecordF4 : 2 * kTableRecordF4) * sizeof(float4);
+        const size_t rec_bytes = (size_t)(sur ? kRecordF4 : (overlap ? 2 : 1) * kTableRecordF4) * sizeof(float4);
         unsigned long long rec_cap = cap * per_packet;
         if (rec_cap < 4 * margin) rec_cap = 4 * margin;
         if (!ctx->d_wave) CK(ctx, cudaMalloc(&ctx->d_wave, sizeof(WaveCtl)));
         if (ctx->wave_cap < cap) {
             cudaFree(ctx->d_susp);
-            cudaFree(ctx->d_res);
             ctx->d_susp = ctx->d_res = nullptr;
             ctx->wave_cap = 0;
-            cudaError_t e = cudaMalloc(&ctx->d_susp, (size_t)cap * kStateF4 * sizeof(float4));
-            if (e == cudaSuccess) e = cudaMalloc(&ctx->d_res, (size_t)cap * kStateF4 * sizeof(float4));
+            const cudaError_t e = cudaMalloc(&ctx->d_susp, 2 * (size_t)cap * kStateF4 * sizeof(float4));
             if (e != cudaSuccess) {
                 (void)cudaGetLastError();
                 return fail(ctx, MCRT_E_NOMEM, "mcrt_launch_packets: surrogate packet buffers: %s", cudaGetErrorString(e));
             }
+            ctx->d_res = ctx->d_susp + (size_t)cap * kStateF4;
             ctx->wave_cap = cap;
         }
         if (ctx->rec_bytes < (size_t)rec_cap * rec_bytes) {
@@ -829,9 +863,6 @@ static mcrt_status launch_one(mcrt_ctx* ctx, const mcrt_launch_desc* d, mcrt_sta
         P.sur.resume = ctx->d_res;
         int n_rounds = 0;
         float ms = 0.f, kms[3] = {0.f, 0.f, 0.f};
-        // overlap of a round's tally with the next transport is opt-in: measured slower on the
-        // disk (the latency-bound transport slows down under the tally's DRAM traffic)
-        const bool overlap = !sur && d->tally_blocks_per_sm > 0;
         if (overlap && !ctx->tally_stream) {
             int lo = 0, hi = 0;
             CK(ctx, cudaDeviceGetStreamPriorityRange(&lo, &hi));
@@ -1048,13 +1079,9 @@ mcrt_status mcrt_destroy(mcrt_ctx* ctx) {
     if (!ctx) return MCRT_OK;
     free_tables(ctx);
     cudaFree(ctx->d_cells);
-    cudaFree(ctx->d_patches);
     cudaFree(ctx->d_cdf);
-    cudaFree(ctx->d_block_sums);
-    cudaFree(ctx->d_guide);
     cudaFree(ctx->d_S);
     cudaFree(ctx->d_absorbed);
-    cudaFree(ctx->d_work);
     free_wave(ctx);
     if (ctx->tally_stream) cudaStreamDestroy(ctx->tally_stream);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
