@@ -133,9 +133,9 @@ __device__ V3<float> iso_unit(float ua, float ub) {
     return V3<float>{st * cp, st * sp, ct};
 }
 
-// Training batch of step step0 + *iter: inputs (zero-padded to 16, BF16) and targets.
+// Training batch of step step0 + *iter: inputs and targets.
 __global__ void k_gen_batch(LabelTables T, unsigned seed, unsigned step0, const unsigned* __restrict__ iter, int B,
-                            bf16* __restrict__ X, float* __restrict__ Y) {
+                            float* __restrict__ X, float* __restrict__ Y) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= B) return;
     const unsigned step = step0 + *iter;
@@ -144,7 +144,7 @@ __global__ void k_gen_batch(LabelTables T, unsigned seed, unsigned step0, const 
     const V3<float> ni = iso_unit(u0.a, u0.b), ns = iso_unit(u0.c, u0.d);
     const float s = 2.f * u1.a - 1.f;
     const float in[kIn] = {ni.x, ni.y, ni.z, ns.x, ns.y, ns.z, s};
-    mlp::store_input_row(X + (size_t)i * kInPad, in);
+    for (int c = 0; c < kIn; ++c) X[(size_t)i * kIn + c] = in[c];
     float out[kOut];
     surrogate_label(T, ni, ns, s, out);
     for (int c = 0; c < kOut; ++c) Y[(size_t)i * kOut + c] = out[c];
@@ -160,150 +160,272 @@ __global__ void k_labels(LabelTables T, int n, const float* __restrict__ in, flo
     for (int c = 0; c < kOut; ++c) out[(size_t)i * kOut + c] = o[c];
 }
 
-__global__ void k_pack_inputs(int n, const float* __restrict__ in, bf16* __restrict__ X) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float u[kIn];
-    for (int c = 0; c < kIn; ++c) u[c] = in[(size_t)i * kIn + c];
-    mlp::store_input_row(X + (size_t)i * kInPad, u);
-}
-
 // ---------------------------------------------------------------------------------
-// BF16 tensor-core GEMM with fused epilogues:  C[m][n] = sum_k A(m,k) B(k,n)
-//   A(m,k) = a_t ? A[k*lda + m] : A[m*lda + k]
-//   B(k,n) = b_kn ? B[k*ldb + n] : B[n*ldb + k]
-// Block tile 64x64x32, 4 warps of 32x32, mma.sync.m16n8k16 (BF16 in, FP32 accumulate).
+// Forward pass, loss and backward pass of a batch in one kernel.  BF16 operands, FP32
+// accumulation (mma.sync m16n8k16); activations, the output gradient and every hidden layer's
+// gradient are rounded to BF16, pre-activations stay in FP32.
+//
+// A block takes tiles of 16 MT rows through all layers: weights (119 kB) and activations in
+// shared memory, the pre-activations in the registers of the warp that owns their 16 columns,
+// which also owns them on the way back.  A layer's gradient overwrites its activations.  The
+// weight gradients of a tile are added to the result with FP32 reductions of two columns.
+//
+// What bounds it: at a tile per SM the chain of ten small products (22 us for 2048 rows), at many
+// tiles the shared-memory reads of the operands (216 us for 65536 rows).  A gradient call, host
+// arrays to host arrays, against one launch per product and epilogue with every operand through
+// memory (25 dependent launches): 2048 rows 88 us (400), 8192 119 us (552), 2^20 3.8 ms (53.9);
+// a training step of 1024 rows 45 us (284), of 8192 70 us (439).
 // ---------------------------------------------------------------------------------
-enum { EPI_HIDDEN = 0, EPI_OUT = 1, EPI_DX = 2, EPI_DW = 3 };
-
-struct GemmArgs {
-    int M, N, K;
-    const bf16* A;
-    int lda, a_t;
-    const bf16* B;
-    int ldb, b_kn;
-    const float* bias;    // HIDDEN, OUT
-    float* Zout;          // HIDDEN: pre-activation; OUT: output; DW: gradient
-    int ldz;
-    bf16* Hout;           // HIDDEN: SiLU(Z); DX: dZ of the previous layer
-    int ldh;
-    const float* Zprev;   // DX: pre-activation of the previous layer
-};
-
-constexpr int kTM = 64, kTN = 64, kTK = 32, kPadK = 40;
-
-__device__ __forceinline__ void mma_bf16(float c[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
-                                         unsigned b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 __device__ __forceinline__ float silu_f(float z) { return mlp::silu(z); }
 __device__ __forceinline__ float silu_grad_f(float z) { return mlp::silu_grad(z); }
 
-template <int EPI> __global__ void __launch_bounds__(128) k_gemm(const GemmArgs g) {
-    __shared__ __align__(16) bf16 As[kTM][kPadK];
-    __shared__ __align__(16) bf16 Bs[kTN][kPadK];
-    const int m0 = blockIdx.y * kTM, n0 = blockIdx.x * kTN;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    const int gr = lane >> 2, tc = lane & 3;
-    float acc[2][4][4];
-    for (int i = 0; i < 2; ++i)
-        for (int j = 0; j < 4; ++j)
-            for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-    const bf16 zero = __float2bfloat16(0.f);
-    // weight gradients split K (the batch) over gridDim.z blocks, which add their
-    // partial sums to the zeroed gradient; the other epilogues take the whole K
-    int kb = 0, ke = g.K;
-    if (EPI == EPI_DW && gridDim.z > 1) {
-        const int per = ((g.K + gridDim.z - 1) / gridDim.z + kTK - 1) / kTK * kTK;
-        kb = blockIdx.z * per;
-        ke = kb + per < g.K ? kb + per : g.K;
-    }
-    for (int k0 = kb; k0 < ke; k0 += kTK) {
-        for (int i = tid; i < kTM * kTK; i += blockDim.x) {
-            const int mm = i / kTK, kk = i % kTK, m = m0 + mm, k = k0 + kk;
-            bf16 v = zero;
-            if (m < g.M && k < ke) v = g.a_t ? g.A[(size_t)k * g.lda + m] : g.A[(size_t)m * g.lda + k];
-            As[mm][kk] = v;
-        }
-        for (int i = tid; i < kTN * kTK; i += blockDim.x) {
-            const int nn = i / kTK, kk = i % kTK, n = n0 + nn, k = k0 + kk;
-            bf16 v = zero;
-            if (n < g.N && k < ke) v = g.b_kn ? g.B[(size_t)k * g.ldb + n] : g.B[(size_t)n * g.ldb + k];
-            Bs[nn][kk] = v;
-        }
-        __syncthreads();
-        for (int ks = 0; ks < kTK; ks += 16) {
-            unsigned a[2][4], b[4][2];
-            for (int mt = 0; mt < 2; ++mt) {
-                const int r = wm + mt * 16 + gr, c = ks + tc * 2;
-                a[mt][0] = *reinterpret_cast<const unsigned*>(&As[r][c]);
-                a[mt][1] = *reinterpret_cast<const unsigned*>(&As[r + 8][c]);
-                a[mt][2] = *reinterpret_cast<const unsigned*>(&As[r][c + 8]);
-                a[mt][3] = *reinterpret_cast<const unsigned*>(&As[r + 8][c + 8]);
-            }
-            for (int nt = 0; nt < 4; ++nt) {
-                const int n = wn + nt * 8 + gr, c = ks + tc * 2;
-                b[nt][0] = *reinterpret_cast<const unsigned*>(&Bs[n][c]);
-                b[nt][1] = *reinterpret_cast<const unsigned*>(&Bs[n][c + 8]);
-            }
-            for (int mt = 0; mt < 2; ++mt)
-                for (int nt = 0; nt < 4; ++nt)
-                    mma_bf16(acc[mt][nt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b[nt][0], b[nt][1]);
-        }
-        __syncthreads();
-    }
-    // epilogue: c0,c1 at (row gr, cols 2tc, 2tc+1), c2,c3 at row gr + 8
-    for (int mt = 0; mt < 2; ++mt)
-        for (int nt = 0; nt < 4; ++nt)
-            for (int h = 0; h < 2; ++h)
-                for (int e = 0; e < 2; ++e) {
-                    const int m = m0 + wm + mt * 16 + gr + h * 8, n = n0 + wn + nt * 8 + tc * 2 + e;
-                    if (m >= g.M || n >= g.N) continue;
-                    const float v = acc[mt][nt][h * 2 + e];
-                    if (EPI == EPI_HIDDEN) {
-                        const float z = v + g.bias[n];
-                        g.Zout[(size_t)m * g.ldz + n] = z;
-                        g.Hout[(size_t)m * g.ldh + n] = __float2bfloat16(silu_f(z));
-                    } else if (EPI == EPI_OUT) {
-                        g.Zout[(size_t)m * g.ldz + n] = v + g.bias[n];
-                    } else if (EPI == EPI_DX) {
-                        g.Hout[(size_t)m * g.ldh + n] = __float2bfloat16(v * silu_grad_f(g.Zprev[(size_t)m * g.ldz + n]));
-                    } else {
-                        if (gridDim.z > 1)
-                            atomicAdd(&g.Zout[(size_t)m * g.ldz + n], v);
-                        else
-                            g.Zout[(size_t)m * g.ldz + n] = v;
-                    }
-                }
+constexpr int kPassThreads = 256, kPassWarps = kPassThreads / 32;
+constexpr int kLdX = mlp::kLd0, kLdH = mlp::kLdH, kLdY = 40;  // row strides (elements), free of bank conflicts
+constexpr int kOutMma = 32;                                  // output columns as a K of the products
+// weights in shared memory: element offset and row stride of layer l (layer 4 has 32 rows, 8 of zeros)
+__host__ __device__ constexpr int pass_w(int l) { return l == 0 ? 0 : kHid * kLdX + (l - 1) * kHid * kLdH; }
+__host__ __device__ constexpr int pass_ld(int l) { return l == 0 ? kLdX : kLdH; }
+constexpr int kPassW = pass_w(kLayers - 1) + kOutMma * kLdH;
+constexpr size_t pass_smem(int mt) {
+    return sizeof(bf16) * (size_t)(kPassW + 16 * mt * (kLdX + 4 * kLdH + kLdY)) + kPassWarps * sizeof(double);
+}
+static_assert(kHid == 16 * kPassWarps, "a warp owns 16 columns of a hidden layer");
+
+struct LossWeights {
+    float w[kOut];
+};
+
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+template <int N> __device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void ldsm_x4_t(unsigned a, unsigned& r0, unsigned& r1, unsigned& r2, unsigned& r3) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(a)
+                 : "memory");
 }
 
-template <int EPI> cudaError_t gemm(const GemmArgs& g, cudaStream_t s) {
-    (void)cudaGetLastError();
-    dim3 grid((g.N + kTN - 1) / kTN, (g.M + kTM - 1) / kTM);
-    // weight gradients (small M x N, K = the batch): split K so that the GPU fills;
-    // the output (d_grads) is zeroed before the backward pass
-    if (EPI == EPI_DW) {
-        int z = 256 / (int)(grid.x * grid.y);
-        const int kmax = (g.K + 4 * kTK - 1) / (4 * kTK);  // at least four k-tiles per block
-        z = z < kmax ? z : kmax;
-        grid.z = z > 1 ? z : 1;
+template <int MT>
+__global__ void __launch_bounds__(kPassThreads, 1)
+    k_pass(int B, const float* __restrict__ in, const float* __restrict__ target, const LossWeights lw,
+           const bf16* __restrict__ wbf, const float* __restrict__ params, float* __restrict__ grads,
+           double* __restrict__ loss, const unsigned* __restrict__ iter) {
+    constexpr int R = 16 * MT;
+    extern __shared__ __align__(16) unsigned char pass_sm[];
+    bf16* const ws = reinterpret_cast<bf16*>(pass_sm);
+    bf16* const xs = ws + kPassW;
+    bf16* const hs = xs + R * kLdX;
+    bf16* const ys = hs + 4 * R * kLdH;
+    double* const part = reinterpret_cast<double*>(ys + R * kLdY);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gr = lane >> 2, tc = lane & 3;
+    // ldmatrix rows and columns of this lane.  A operand with k contiguous, or its transpose from
+    // rows of k; B operand with k contiguous (16 columns), or from rows of k
+    const int a_row = lane & 15, a_col = (lane >> 4) * 8;
+    const int at_row = (lane & 7) + (lane >> 4) * 8, at_col = ((lane >> 3) & 1) * 8;
+    const int b_row = (lane & 7) + (lane >> 4) * 8, b_col = ((lane >> 3) & 1) * 8;
+    const int bt_row = (lane & 7) + ((lane >> 3) & 1) * 8, bt_col = (lane >> 4) * 8;
+    const unsigned ws_a = mlp::smem_addr(ws), xs_a = mlp::smem_addr(xs), hs_a = mlp::smem_addr(hs),
+                   ys_a = mlp::smem_addr(ys);
+    // weights: one group of copies per layer, waited for when the layer is reached
+#pragma unroll
+    for (int l = 0; l < kLayers; ++l) {
+        const int per_row = layer_in(l) / 8, n = layer_out(l) * per_row;
+        for (int i = tid; i < n; i += kPassThreads)
+            cp_async16(ws_a + (unsigned)(pass_w(l) + i / per_row * pass_ld(l) + i % per_row * 8) * 2,
+                       wbf + wbf_offset(l) + i * 8);
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    k_gemm<EPI><<<grid, 128, 0, s>>>(g);
-    return cudaGetLastError();
+    const bf16 zero = __float2bfloat16(0.f);
+    for (int i = tid; i < (kOutMma - kOutPad) * kLdH; i += kPassThreads)
+        ws[pass_w(kLayers - 1) + kOutPad * kLdH + i] = zero;
+    for (int i = tid; i < R * kLdY; i += kPassThreads) ys[i] = zero;
+    const float scale = 2.f / ((float)B * (float)kOut);
+    double lsum = 0.0;
+    const int n_tiles = (B + R - 1) / R;
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int row0 = tile * R;
+        __syncthreads();  // the tile before is done with the input rows
+        for (int i = tid; i < R; i += kPassThreads) {
+            float u[kIn];
+            for (int c = 0; c < kIn; ++c) u[c] = row0 + i < B ? in[(size_t)(row0 + i) * kIn + c] : 0.f;
+            mlp::store_input_row(xs + i * kLdX, u);
+        }
+        // ---- forward: z = h W^T + b, h = SiLU(z)
+        float z[4][MT][2][4];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            if (l == 0) cp_async_wait<4>();
+            if (l == 1) cp_async_wait<3>();
+            if (l == 2) cp_async_wait<2>();
+            if (l == 3) cp_async_wait<1>();
+            __syncthreads();
+            float acc[MT][2][4] = {};
+            const unsigned src = l == 0 ? xs_a : hs_a + (unsigned)((l - 1) * R * kLdH * 2);
+            const int ld = l == 0 ? kLdX : kLdH;
+#pragma unroll
+            for (int ks = 0; ks < layer_in(l); ks += 16) {
+                unsigned b[4];
+                mlp::ldsm_x4_fenced(ws_a + (unsigned)(pass_w(l) + (warp * 16 + b_row) * pass_ld(l) + ks + b_col) * 2, b[0],
+                                    b[1], b[2], b[3]);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    unsigned a[4];
+                    mlp::ldsm_x4_fenced(src + (unsigned)((mt * 16 + a_row) * ld + ks + a_col) * 2, a[0], a[1], a[2], a[3]);
+                    mlp::mma16816(acc[mt][0], a, b[0], b[1]);
+                    mlp::mma16816(acc[mt][1], a, b[2], b[3]);
+                }
+            }
+            const float* const bias = params + layer_offset(l) + kHid * layer_in(l);
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                const int n = warp * 16 + nt * 8 + tc * 2;
+                const float b0 = __ldg(bias + n), b1 = __ldg(bias + n + 1);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float z0 = acc[mt][nt][h * 2] + b0, z1 = acc[mt][nt][h * 2 + 1] + b1;
+                        z[l][mt][nt][h * 2] = z0;
+                        z[l][mt][nt][h * 2 + 1] = z1;
+                        *reinterpret_cast<unsigned*>(hs + (l * R + mt * 16 + gr + h * 8) * kLdH + n) =
+                            mlp::pack_bf16(silu_f(z0), silu_f(z1));
+                    }
+            }
+        }
+        cp_async_wait<0>();
+        __syncthreads();
+        // ---- output, loss and dY = 2 w (Y - T) / (B * 20): one 16 x 8 tile per warp
+        if (warp < 3 * MT) {
+            const int mt = warp / 3, nt = warp % 3;
+            float acc[4] = {};
+#pragma unroll
+            for (int ks = 0; ks < kHid; ks += 16) {
+                unsigned a[4], b0, b1;
+                mlp::ldsm_x4_fenced(hs_a + (unsigned)((3 * R + mt * 16 + a_row) * kLdH + ks + a_col) * 2, a[0], a[1], a[2],
+                                    a[3]);
+                mlp::ldsm_x2(ws_a + (unsigned)(pass_w(4) + (nt * 8 + (lane & 7)) * kLdH + ks + b_col) * 2, b0, b1);
+                mlp::mma16816(acc, a, b0, b1);
+            }
+            const float* const bias = params + layer_offset(4) + kOutPad * kHid;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = mt * 16 + gr + h * 8, o = nt * 8 + tc * 2;
+                float d[2] = {0.f, 0.f};
+                if (row0 + r < B && o < kOut) {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float y = acc[h * 2 + e] + __ldg(bias + o + e);
+                        const float res = y - target[(size_t)(row0 + r) * kOut + o + e];
+                        lsum += (double)(lw.w[o + e] * res * res);
+                        d[e] = scale * lw.w[o + e] * res;
+                    }
+                }
+                *reinterpret_cast<unsigned*>(ys + r * kLdY + o) = mlp::pack_bf16(d[0], d[1]);
+            }
+        }
+        __syncthreads();
+        // ---- backward
+#pragma unroll
+        for (int l = kLayers - 1; l >= 0; --l) {
+            constexpr int kLast = kLayers - 1;
+            const int no = layer_out(l), ni = layer_in(l);
+            const bf16* const dz = l == kLast ? ys : hs + l * R * kLdH;
+            const unsigned dz_a = l == kLast ? ys_a : hs_a + (unsigned)(l * R * kLdH * 2);
+            const int dz_ld = l == kLast ? kLdY : kLdH;
+            const unsigned in_a = l == 0 ? xs_a : hs_a + (unsigned)((l - 1) * R * kLdH * 2);
+            const int in_ld = l == 0 ? kLdX : kLdH;
+            float* const gW = grads + layer_offset(l);
+            // dW = dZ^T H: 16 x 16 tiles, a row of them per warp (layer 4: a column of two)
+            const int tiles = l == kLast ? 2 : ni / 16;
+            for (int t = 0; t < tiles; ++t) {
+                const int m0 = (l == kLast ? t : warp) * 16, n0 = (l == kLast ? warp : t) * 16;
+                float acc[2][4] = {};
+#pragma unroll
+                for (int ks = 0; ks < R; ks += 16) {
+                    unsigned a[4], b[4];
+                    ldsm_x4_t(dz_a + (unsigned)((ks + at_row) * dz_ld + m0 + at_col) * 2, a[0], a[1], a[2], a[3]);
+                    ldsm_x4_t(in_a + (unsigned)((ks + bt_row) * in_ld + n0 + bt_col) * 2, b[0], b[1], b[2], b[3]);
+                    mlp::mma16816(acc[0], a, b[0], b[1]);
+                    mlp::mma16816(acc[1], a, b[2], b[3]);
+                }
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int m = m0 + gr + h * 8, n = n0 + nt * 8 + tc * 2;
+                        if (l == 0) {
+                            // a master weight feeds the column of the high parts and that of the low parts
+                            for (int e = 0; e < 2; ++e)
+                                if (n + e < 2 * kIn)
+                                    atomicAdd(gW + m * kInPad + (n + e < kIn ? n + e : n + e - kIn), acc[nt][h * 2 + e]);
+                        } else if (m < no) {
+                            atomicAdd(reinterpret_cast<float2*>(gW + m * ni + n),
+                                      make_float2(acc[nt][h * 2], acc[nt][h * 2 + 1]));
+                        }
+                    }
+            }
+            // db = column sums of dZ
+            if (tid < no) {
+                float sum = 0.f;
+#pragma unroll 8
+                for (int r = 0; r < R; ++r) sum += __bfloat162float(dz[r * dz_ld + tid]);
+                atomicAdd(gW + no * ni + tid, sum);
+            }
+            if (l == 0) break;
+            // dZ of the layer below = (dZ W) SiLU'(z)
+            float acc[MT][2][4] = {};
+#pragma unroll
+            for (int ks = 0; ks < (l == kLast ? kOutMma : kHid); ks += 16) {
+                unsigned b[4];
+                ldsm_x4_t(ws_a + (unsigned)(pass_w(l) + (ks + bt_row) * kLdH + warp * 16 + bt_col) * 2, b[0], b[1], b[2],
+                          b[3]);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    unsigned a[4];
+                    mlp::ldsm_x4_fenced(dz_a + (unsigned)((mt * 16 + a_row) * dz_ld + ks + a_col) * 2, a[0], a[1], a[2],
+                                        a[3]);
+                    mlp::mma16816(acc[mt][0], a, b[0], b[1]);
+                    mlp::mma16816(acc[mt][1], a, b[2], b[3]);
+                }
+            }
+            __syncthreads();  // the activations of the layer below have been read
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int r = mt * 16 + gr + h * 8, n = warp * 16 + nt * 8 + tc * 2;
+                        const bool live = row0 + r < B;
+                        const float d0 = acc[mt][nt][h * 2] * silu_grad_f(z[l - 1][mt][nt][h * 2]);
+                        const float d1 = acc[mt][nt][h * 2 + 1] * silu_grad_f(z[l - 1][mt][nt][h * 2 + 1]);
+                        *reinterpret_cast<unsigned*>(hs + ((l - 1) * R + r) * kLdH + n) =
+                            live ? mlp::pack_bf16(d0, d1) : 0u;
+                    }
+            __syncthreads();
+        }
+    }
+    for (int off = 16; off > 0; off >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, off);
+    if (lane == 0) part[warp] = lsum;
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < kPassWarps; ++w) lsum += part[w];
+        atomicAdd(loss + (iter ? *iter : 0u), lsum / ((double)B * kOut));
+    }
 }
 
 // ---------------------------------------------------------------------------------
 // FP32 mode of the training passes, for gradient checks at FP32 accuracy: the same
 // layers and fused epilogues with FP32 operands and activations on the FP32 pipe (no
-// BF16 rounding anywhere), C[m][n] = sum_k A(m,k) B(k,n) with the index rules of
-// GemmArgs.  Block tile 64x64x16, 256 threads of 4x4 outputs each.
+// BF16 rounding anywhere), C[m][n] = sum_k A(m,k) B(k,n),
+//   A(m,k) = a_t ? A[k*lda + m] : A[m*lda + k],  B(k,n) = b_kn ? B[k*ldb + n] : B[n*ldb + k].
+// Block tile 64x64x16, 256 threads of 4x4 outputs each.
 // ---------------------------------------------------------------------------------
+enum { EPI_HIDDEN = 0, EPI_OUT = 1, EPI_DX = 2, EPI_DW = 3 };
+
 struct GemmArgs32 {
     int M, N, K;
     const float* A;
@@ -398,7 +520,7 @@ __global__ void k_pack_inputs32(int n, const float* __restrict__ in, float* __re
     for (int c = 0; c < kInPad; ++c) X[(size_t)i * kInPad + c] = c < kIn ? in[(size_t)i * kIn + c] : 0.f;
 }
 
-// dY = 2 w (Y - T) / (B * 20) in FP32 and the loss sum (the FP32 twin of k_loss_grad).
+// dY = 2 w (Y - T) / (B * 20) in FP32 and the loss sum.
 __global__ void k_loss_grad32(int B, const float* __restrict__ Y, const float* __restrict__ T,
                               const float* __restrict__ w, float* __restrict__ dY, double* __restrict__ loss) {
     __shared__ double part[256];
@@ -429,42 +551,6 @@ __global__ void k_colsum32(int B, int N, const float* __restrict__ dZ, float* __
     if (n >= N) return;
     float s = 0.f;
     for (int b = blockIdx.y; b < B; b += gridDim.y) s += dZ[(size_t)b * N + n];
-    atomicAdd(&db[n], s);
-}
-
-// dY = 2 w (Y - T) / (B * 20) (BF16, zero in the padding columns) and the loss sum,
-// added to loss[*iter] (loss[0] without an iteration counter).
-__global__ void k_loss_grad(int B, const float* __restrict__ Y, const float* __restrict__ T,
-                            const float* __restrict__ w, bf16* __restrict__ dY, double* __restrict__ loss,
-                            const unsigned* __restrict__ iter) {
-    __shared__ double part[256];
-    double acc = 0.0;
-    const float scale = 2.f / ((float)B * (float)kOut);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < B * kOutPad; i += gridDim.x * blockDim.x) {
-        const int b = i / kOutPad, o = i % kOutPad;
-        float d = 0.f;
-        if (o < kOut) {
-            const float r = Y[(size_t)b * kOutPad + o] - T[(size_t)b * kOut + o];
-            acc += (double)(w[o] * r * r);
-            d = scale * w[o] * r;
-        }
-        dY[i] = __float2bfloat16(d);
-    }
-    part[threadIdx.x] = acc;
-    __syncthreads();
-    for (int off = blockDim.x / 2; off > 0; off >>= 1) {
-        if (threadIdx.x < off) part[threadIdx.x] += part[threadIdx.x + off];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(loss + (iter ? *iter : 0u), part[0] / ((double)B * kOut));
-}
-
-// db[n] = sum over rows of dZ[b][n] (BF16 input, FP32 output).
-__global__ void k_colsum(int B, int N, const bf16* __restrict__ dZ, float* __restrict__ db) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float s = 0.f;
-    for (int b = blockIdx.y; b < B; b += gridDim.y) s += __bfloat162float(dZ[(size_t)b * N + n]);
     atomicAdd(&db[n], s);
 }
 
@@ -505,16 +591,6 @@ __global__ void k_pack_weights(const float* __restrict__ p, bf16* __restrict__ w
             wbf[wbf_offset(l) + i] = __float2bfloat16(v);
         }
     }
-}
-
-// Layer-0 weight gradient: a master weight feeds both the hi and the lo column, so
-// its gradient is the sum of the two; the unused columns get zero.
-__global__ void k_fold_l0(float* __restrict__ g) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= kHid) return;
-    float* row = g + (size_t)o * kInPad;
-    for (int c = 0; c < kIn; ++c) row[c] += row[c + kIn];
-    for (int c = kIn; c < kInPad; ++c) row[c] = 0.f;
 }
 
 // Inference image (layout in mcrt_mlp_infer.cuh) from the FP32 parameters.
@@ -747,17 +823,6 @@ __global__ void __launch_bounds__(kInferBlock) k_distill_kext(const unsigned cha
 // ---------------------------------------------------------------------------------
 // host side: the surrogate object
 // ---------------------------------------------------------------------------------
-struct SurrogateBuffers {
-    int B = 0;
-    bf16* x0 = nullptr;
-    float* z[4] = {nullptr, nullptr, nullptr, nullptr};
-    bf16* h[4] = {nullptr, nullptr, nullptr, nullptr};
-    float* y = nullptr;
-    float* t = nullptr;
-    bf16* dy = nullptr;
-    bf16* dz[2] = {nullptr, nullptr};
-};
-
 }  // namespace mcrt
 
 using namespace mcrt;
@@ -774,9 +839,10 @@ struct mcrt_surrogate {
     float* d_w = nullptr;  // loss weights [20]
     bf16* d_wbf = nullptr;
     double* d_loss = nullptr;
-    float* d_in = nullptr;  // staging of user inputs
+    float* d_in = nullptr;  // inputs of a user or of a training step
     size_t in_cap = 0;
-    SurrogateBuffers buf;
+    float* d_t = nullptr;  // targets
+    size_t t_cap = 0;
     unsigned seed = 0;
     long long step = 0;
     unsigned char* d_image = nullptr;  // inference image of the current parameters
@@ -796,142 +862,47 @@ namespace {
         }                                                                                               \
     } while (0)
 
-void free_buffers(SurrogateBuffers& b) {
-    cudaFree(b.x0);
-    for (int i = 0; i < 4; ++i) {
-        cudaFree(b.z[i]);
-        cudaFree(b.h[i]);
-    }
-    cudaFree(b.y);
-    cudaFree(b.t);
-    cudaFree(b.dy);
-    cudaFree(b.dz[0]);
-    cudaFree(b.dz[1]);
-    b = SurrogateBuffers{};
-}
-
-cudaError_t ensure_buffers(SurrogateBuffers& b, int B) {
-    if (b.B >= B) return cudaSuccess;
-    free_buffers(b);
-    cudaError_t e = cudaMalloc(&b.x0, (size_t)B * kInPad * sizeof(bf16));
-    for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
-        e = cudaMalloc(&b.z[i], (size_t)B * kHid * sizeof(float));
-        if (e == cudaSuccess) e = cudaMalloc(&b.h[i], (size_t)B * kHid * sizeof(bf16));
-    }
-    if (e == cudaSuccess) e = cudaMalloc(&b.y, (size_t)B * kOutPad * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&b.t, (size_t)B * kOut * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&b.dy, (size_t)B * kOutPad * sizeof(bf16));
-    if (e == cudaSuccess) e = cudaMalloc(&b.dz[0], (size_t)B * kHid * sizeof(bf16));
-    if (e == cudaSuccess) e = cudaMalloc(&b.dz[1], (size_t)B * kHid * sizeof(bf16));
-    if (e != cudaSuccess) {
-        free_buffers(b);
-        return e;
-    }
-    b.B = B;
-    return cudaSuccess;
+// Room for n rows of inputs, and of targets.
+mcrt_status ensure(float*& d, size_t& cap, size_t bytes) {
+    if (cap >= bytes) return MCRT_OK;
+    cudaFree(d);
+    d = nullptr;
+    cap = 0;
+    SK(cudaMalloc(&d, bytes));
+    cap = bytes;
+    return MCRT_OK;
 }
 
 LabelTables tables_of(const mcrt_surrogate* s) {
     return LabelTables{s->d_bins, s->d_kext, s->n_bins, s->n_theta, s->n_ktheta};
 }
 
-// Forward pass on buf.x0 rows [0, B): hidden activations and the output buf.y.
-mcrt_status forward(mcrt_surrogate* s, int B) {
-    SurrogateBuffers& b = s->buf;
-    for (int l = 0; l < kLayers; ++l) {
-        GemmArgs g{};
-        g.M = B;
-        g.N = layer_out(l);
-        g.K = layer_in(l);
-        g.A = l == 0 ? b.x0 : b.h[l - 1];
-        g.lda = layer_in(l);
-        g.a_t = 0;
-        g.B = s->d_wbf + wbf_offset(l);
-        g.ldb = layer_in(l);
-        g.b_kn = 0;
-        g.bias = s->d_params + layer_offset(l) + layer_out(l) * layer_in(l);
-        if (l < kLayers - 1) {
-            g.Zout = b.z[l];
-            g.ldz = kHid;
-            g.Hout = b.h[l];
-            g.ldh = kHid;
-            SK(gemm<EPI_HIDDEN>(g, s->stream));
-        } else {
-            g.Zout = b.y;
-            g.ldz = kOutPad;
-            SK(gemm<EPI_OUT>(g, s->stream));
-        }
-    }
-    return MCRT_OK;
-}
-
-// Backward pass after forward() and the loss gradient in buf.dy: gradients of all
-// parameters into d_grads (FP32).
-mcrt_status backward(mcrt_surrogate* s, int B) {
-    SurrogateBuffers& b = s->buf;
+// Loss and gradients of the B rows in d_in and d_t: gradients of all parameters into d_grads
+// (FP32), the loss added to loss[*iter] (loss[0] without an iteration counter).  Tiles of 16
+// rows while there is an SM for each (a training step of 1024 rows 45 us, 47 with 32), else of
+// 32, which add the weight gradients half as often (2^16 rows: 0.31 ms, 0.45 with 16).
+mcrt_status pass(mcrt_surrogate* s, int B, const LossWeights& w, double* loss, const unsigned* iter) {
     SK(cudaMemsetAsync(s->d_grads, 0, sizeof(float) * kParams, s->stream));
-    const bf16* dZ = b.dy;  // gradient w.r.t. the pre-activation of layer l
-    int cur = 0;
-    for (int l = kLayers - 1; l >= 0; --l) {
-        const int no = layer_out(l), ni = layer_in(l);
-        const bf16* Hin = l == 0 ? b.x0 : b.h[l - 1];
-        // dW = dZ^T Hin : M = no, N = ni, K = B
-        GemmArgs gw{};
-        gw.M = no;
-        gw.N = ni;
-        gw.K = B;
-        gw.A = dZ;
-        gw.lda = no;
-        gw.a_t = 1;
-        gw.B = Hin;
-        gw.ldb = ni;
-        gw.b_kn = 1;
-        gw.Zout = s->d_grads + layer_offset(l);
-        gw.ldz = ni;
-        SK(gemm<EPI_DW>(gw, s->stream));
-        // db = column sums of dZ
-        {
-            (void)cudaGetLastError();
-            const dim3 grid((no + 127) / 128, 64);
-            k_colsum<<<grid, 128, 0, s->stream>>>(B, no, dZ, s->d_grads + layer_offset(l) + no * ni);
-            SK(cudaGetLastError());
-        }
-        if (l == 0) {
-            k_fold_l0<<<1, kHid, 0, s->stream>>>(s->d_grads + layer_offset(0));
-            SK(cudaGetLastError());
-            break;
-        }
-        // dZ_{l-1} = (dZ W) * SiLU'(Z_{l-1}) : M = B, N = ni, K = no
-        GemmArgs gx{};
-        gx.M = B;
-        gx.N = ni;
-        gx.K = no;
-        gx.A = dZ;
-        gx.lda = no;
-        gx.a_t = 0;
-        gx.B = s->d_wbf + wbf_offset(l);
-        gx.ldb = ni;
-        gx.b_kn = 1;
-        gx.Zprev = b.z[l - 1];
-        gx.ldz = kHid;
-        gx.Hout = b.dz[cur];
-        gx.ldh = kHid;
-        SK(gemm<EPI_DX>(gx, s->stream));
-        dZ = b.dz[cur];
-        cur ^= 1;
+    const int small = B <= 16 * s->n_sm, rows = small ? 16 : 32;
+    const int tiles = (B + rows - 1) / rows, grid = tiles < s->n_sm ? tiles : s->n_sm;
+    (void)cudaGetLastError();
+    if (small) {
+        SK(cudaFuncSetAttribute(k_pass<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pass_smem(1)));
+        k_pass<1><<<grid, kPassThreads, pass_smem(1), s->stream>>>(B, s->d_in, s->d_t, w, s->d_wbf, s->d_params,
+                                                                   s->d_grads, loss, iter);
+    } else {
+        SK(cudaFuncSetAttribute(k_pass<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pass_smem(2)));
+        k_pass<2><<<grid, kPassThreads, pass_smem(2), s->stream>>>(B, s->d_in, s->d_t, w, s->d_wbf, s->d_params,
+                                                                   s->d_grads, loss, iter);
     }
+    SK(cudaGetLastError());
     return MCRT_OK;
 }
 
 mcrt_status stage_inputs(mcrt_surrogate* s, const float* in, long long n) {
     const size_t bytes = (size_t)n * kIn * sizeof(float);
-    if (s->in_cap < bytes) {
-        cudaFree(s->d_in);
-        s->d_in = nullptr;
-        s->in_cap = 0;
-        SK(cudaMalloc(&s->d_in, bytes));
-        s->in_cap = bytes;
-    }
+    const mcrt_status st = ensure(s->d_in, s->in_cap, bytes);
+    if (st != MCRT_OK) return st;
     SK(cudaMemcpyAsync(s->d_in, in, bytes, cudaMemcpyDefault, s->stream));
     return MCRT_OK;
 }
@@ -1072,7 +1043,11 @@ mcrt_status mcrt_surrogate_create(mcrt_surrogate** out, const mcrt_ctx* optics, 
 mcrt_status mcrt_surrogate_train(mcrt_surrogate* s, int64_t n_steps, int32_t batch, double lr, double* loss_history) {
     if (!s || n_steps < 0 || batch < 64 || batch > (1 << 20) || n_steps > (1ll << 31))
         return mcrt_fail_noctx(MCRT_E_INVAL, "mcrt_surrogate_train: bad arguments");
-    SK(ensure_buffers(s->buf, batch));
+    {
+        mcrt_status st = ensure(s->d_in, s->in_cap, (size_t)batch * kIn * sizeof(float));
+        if (st == MCRT_OK) st = ensure(s->d_t, s->t_cap, (size_t)batch * kOut * sizeof(float));
+        if (st != MCRT_OK) return st;
+    }
     s->map_valid = false;
     if (n_steps == 0) return MCRT_OK;
     const LabelTables T = tables_of(s);
@@ -1117,15 +1092,14 @@ mcrt_status mcrt_surrogate_train(mcrt_surrogate* s, int64_t n_steps, int32_t bat
     e = cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return done(mcrt_fail_noctx(MCRT_E_CUDA, "mcrt_surrogate_train: %s", cudaGetErrorString(e)));
     mcrt_status st = MCRT_OK;
-    k_gen_batch<<<(batch + 127) / 128, 128, 0, s->stream>>>(T, s->seed, (unsigned)s->step, d_iter, batch, s->buf.x0,
-                                                            s->buf.t);
+    k_gen_batch<<<(batch + 127) / 128, 128, 0, s->stream>>>(T, s->seed, (unsigned)s->step, d_iter, batch, s->d_in,
+                                                            s->d_t);
     if (cudaGetLastError() != cudaSuccess) st = MCRT_E_CUDA;
-    if (st == MCRT_OK) st = forward(s, batch);
     if (st == MCRT_OK) {
-        k_loss_grad<<<256, 256, 0, s->stream>>>(batch, s->buf.y, s->buf.t, s->d_w, s->buf.dy, d_hist, d_iter);
-        if (cudaGetLastError() != cudaSuccess) st = MCRT_E_CUDA;
+        LossWeights w;
+        for (float& v : w.w) v = 1.f;
+        st = pass(s, batch, w, d_hist, d_iter);
     }
-    if (st == MCRT_OK) st = backward(s, batch);
     if (st == MCRT_OK) {
         k_adam<<<128, 256, 0, s->stream>>>(kParams, s->d_params, s->d_grads, s->d_m, s->d_v, d_sched, d_iter, b1, b2,
                                            eps);
@@ -1246,26 +1220,17 @@ mcrt_status mcrt_surrogate_grad(mcrt_surrogate* s, int64_t n, const float* input
         return mcrt_fail_noctx(MCRT_E_INVAL, "mcrt_surrogate_grad: bad arguments");
     mcrt_status st = stage_inputs(s, inputs, n);
     if (st != MCRT_OK) return st;
-    SK(ensure_buffers(s->buf, (int)n));
-    (void)cudaGetLastError();
-    k_pack_inputs<<<(unsigned)((n + 127) / 128), 128, 0, s->stream>>>((int)n, s->d_in, s->buf.x0);
-    SK(cudaGetLastError());
-    SK(cudaMemcpyAsync(s->buf.t, targets, (size_t)n * kOut * sizeof(float), cudaMemcpyDefault, s->stream));
-    std::vector<float> w(kOut, 1.f);
-    if (loss_weights) std::memcpy(w.data(), loss_weights, sizeof(float) * kOut);
-    SK(cudaMemcpyAsync(s->d_w, w.data(), sizeof(float) * kOut, cudaMemcpyHostToDevice, s->stream));
-    st = forward(s, (int)n);
+    st = ensure(s->d_t, s->t_cap, (size_t)n * kOut * sizeof(float));
     if (st != MCRT_OK) return st;
+    SK(cudaMemcpyAsync(s->d_t, targets, (size_t)n * kOut * sizeof(float), cudaMemcpyDefault, s->stream));
+    LossWeights w;
+    for (int o = 0; o < kOut; ++o) w.w[o] = loss_weights ? loss_weights[o] : 1.f;
     SK(cudaMemsetAsync(s->d_loss, 0, sizeof(double), s->stream));
-    k_loss_grad<<<256, 256, 0, s->stream>>>((int)n, s->buf.y, s->buf.t, s->d_w, s->buf.dy, s->d_loss, nullptr);
-    SK(cudaGetLastError());
-    st = backward(s, (int)n);
+    st = pass(s, (int)n, w, s->d_loss, nullptr);
     if (st != MCRT_OK) return st;
     SK(cudaMemcpyAsync(grads, s->d_grads, sizeof(float) * kParams, cudaMemcpyDefault, s->stream));
     double l = 0.0;
     SK(cudaMemcpyAsync(&l, s->d_loss, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
-    std::vector<float> ones(kOut, 1.f);
-    SK(cudaMemcpyAsync(s->d_w, ones.data(), sizeof(float) * kOut, cudaMemcpyHostToDevice, s->stream));
     SK(cudaStreamSynchronize(s->stream));
     if (loss) *loss = l;
     return MCRT_OK;
@@ -1408,7 +1373,7 @@ int64_t mcrt_surrogate_param_count(void) { return kParams; }
 mcrt_status mcrt_surrogate_destroy(mcrt_surrogate* s) {
     if (!s) return MCRT_OK;
     if (s->stream) cudaStreamSynchronize(s->stream);
-    free_buffers(s->buf);
+    cudaFree(s->d_t);
     cudaFree(s->d_bins);
     cudaFree(s->d_kext);
     cudaFree(s->d_params);
