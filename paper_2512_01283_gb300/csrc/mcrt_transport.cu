@@ -524,8 +524,9 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
     const bool lost = !capped && axis < 0;
     const bool want_A = !capped && !lost && kext > T(0);
     const bool want_S = want_A && ks > T(0) && P.n_cam > 0;
+    // cell indices are below 2^31
     const unsigned c32 = pt ? (unsigned)patch_cell(*pt, pk.ix, pk.iy, pk.iz)
-                            : (unsigned)(((long long)pk.iz * job.n(1) + pk.iy) * job.n(0) + pk.ix);
+                            : ((unsigned)pk.iz * job.n(1) + pk.iy) * job.n(0) + pk.ix;
     // converged point: same-cell groups (of the same model) for the aggregated
     // tallies; lanes that leave below are outside actA / actS
     constexpr bool kGroups = round_based(SCAT) ? MCRT_ABS_GROUPS : MCRT_INPLACE_GROUPS;
@@ -564,26 +565,26 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
     bool next_in = true;
     float4 nq = pk.cq, nr = pk.cr;
     if (!scatter_here) {
-        int* ni = axis == 0 ? &nix : (axis == 1 ? &niy : &niz);
         const T na = axis == 0 ? pk.nx : (axis == 1 ? pk.ny : pk.nz);
-        const int nn = pt ? pt->n[axis] : job.n(axis);
-        *ni += na > T(0) ? 1 : -1;
-        next_in = *ni >= 0 && *ni < nn;
-        if (pt) {
-            // within the patch; leaving it is resolved below, once the packet is on the face
-            if (next_in) {
-                const long long c = patch_cell(*pt, nix, niy, niz);
-                nq = __ldg(&job.cells()[2 * c]);
-                nr = __ldg(&job.cells()[2 * c + 1]);
-            }
-        } else {
-            if (!next_in && ((job.periodic() >> axis) & 1)) {
-                // a periodic axis: the packet re-enters on the opposite face
-                face = na > T(0) ? job.lo(axis) : job.lo(axis) + T(nn) * job.d(axis);
-                *ni = na > T(0) ? 0 : nn - 1;
-                next_in = true;
-            }
-            if (next_in) load_cell(job, nix, niy, niz, nq, nr);
+        const bool up = na > T(0);
+        const int nn = pt ? pt->n[axis] : (axis == 0 ? job.n(0) : (axis == 1 ? job.n(1) : job.n(2)));
+        int at = (axis == 0 ? nix : (axis == 1 ? niy : niz)) + (up ? 1 : -1);
+        next_in = (unsigned)at < (unsigned)nn;
+        if (!pt && !next_in && ((job.periodic() >> axis) & 1)) {
+            // a periodic axis: the packet re-enters on the opposite face
+            face = up ? job.lo(axis) : job.lo(axis) + T(nn) * job.d(axis);
+            at = up ? 0 : nn - 1;
+            next_in = true;
+        }
+        nix = axis == 0 ? at : nix;
+        niy = axis == 1 ? at : niy;
+        niz = axis == 2 ? at : niz;
+        // within a patch; leaving it is resolved below, once the packet is on the face
+        if (next_in) {
+            const unsigned c = pt ? (unsigned)patch_cell(*pt, nix, niy, niz)
+                                  : ((unsigned)niz * job.n(1) + niy) * job.n(0) + nix;
+            nq = __ldg(&job.cells()[2 * (size_t)c]);
+            nr = __ldg(&job.cells()[2 * (size_t)c + 1]);
         }
     }
 
