@@ -598,6 +598,7 @@ static void fill_common(const mcrt_launch_desc* d, TransportParams& P) {
     P.stream = d->stream;
     P.roulette_thr = d->roulette_threshold;
     P.roulette_surv = d->roulette_survival > 0.0 ? d->roulette_survival : 1.0;
+    P.roulette_gain = 1.0 / P.roulette_surv;
     P.max_events = d->max_events > 0 ? (d->max_events < 2147483647ll ? d->max_events : 2147483647ll) : 100000;
     P.max_trials = d->max_trials > 0 ? d->max_trials : 1000;
     P.time_budget_ns = d->time_budget_s > 0.0 ? d->time_budget_s * 1e9 : 0.0;

@@ -239,6 +239,18 @@ template <typename T> __device__ __forceinline__ T e1(T x) {
     return t_div(-t_expm1(-x), x);
 }
 
+// The sine and cosine that only media with a circular-retardance element (a3 != 0) need: a function
+// of its own, so that its slow path, with the stack that takes, stays out of the walk of everything
+// else (refined disk's transport 82.1 -> 78.9 ms, plane-parallel slab 383 -> 376 ms).
+template <typename T> struct Pair {
+    T a, b;
+};
+template <typename T> __device__ __noinline__ Pair<T> sincos_apart(T y) {
+    Pair<T> p;
+    t_sincos(y, &p.a, &p.b);
+    return p;
+}
+
 // int_0^1 e^{-(x - i y) s} ds = (re, im)
 template <typename T> __device__ __forceinline__ void e1_complex(T x, T y, T& re, T& im) {
     if (y == T(0)) {
@@ -247,20 +259,18 @@ template <typename T> __device__ __forceinline__ void e1_complex(T x, T y, T& re
         return;
     }
     if (fabs(x) + fabs(y) < T(1e-4)) {
-        re = T(1) - x * T(0.5) + (x * x - y * y) * T(1.0 / 6.0);
-        im = y * T(0.5) - x * y * T(1.0 / 3.0);
+        re = t_fma(msb2(x, x, y, y), T(1.0 / 6.0), t_fma(-x, T(0.5), T(1)));
+        im = msb2(y, T(0.5), t_mul(x, y), T(1.0 / 3.0));
         return;
     }
-    T sh, ch, sy, cy;
-    t_sincos(T(0.5) * y, &sh, &ch);
-    sy = T(2) * sh * ch;
+    const Pair<T> half = sincos_apart(T(0.5) * y);
+    const T sh = half.a, sy = T(2) * sh * half.b;
     const T ex = t_exp(-x);
-    const T nr = -t_expm1(-x) + T(2) * ex * sh * sh;  // 1 - e^{-x} cos y
-    const T ni = ex * sy;                               // e^{-x} sin y
-    const T den = t_rcp(x * x + y * y);
-    re = (nr * x + ni * y) * den;
-    im = (nr * y - ni * x) * den;
-    (void)cy;
+    const T nr = t_fma(T(2) * ex * sh, sh, -t_expm1(-x));  // 1 - e^{-x} cos y
+    const T ni = t_mul(ex, sy);                             // e^{-x} sin y
+    const T den = t_rcp(mad2<kSecond>(x, x, y, y));
+    re = t_mul(mad2(nr, x, ni, y), den);
+    im = t_mul(msb2(nr, y, ni, x), den);
 }
 
 // The coefficients of Y = e^{-M dtau} X.  For |a2 dtau| <= 10 the I-Q block uses the
@@ -286,7 +296,11 @@ template <typename T> __device__ __forceinline__ Decay<T> decay_of(T xa, T xb, T
     }
     d.s3 = T(0);
     d.c3 = T(1);
-    if (ya != T(0)) t_sincos(ya, &d.s3, &d.c3);
+    if (ya != T(0)) {
+        const Pair<T> p = sincos_apart(ya);
+        d.s3 = p.a;
+        d.c3 = p.b;
+    }
     return d;
 }
 

@@ -203,7 +203,7 @@ struct TransportParams {
     double* absorbed;  // [ncell]
     unsigned seed, stream;
     long long pid_begin, pid_end;
-    double roulette_thr, roulette_surv;
+    double roulette_thr, roulette_surv, roulette_gain;  // gain: 1 / surv
     long long max_events;
     int max_trials;
     double time_budget_ns;  // <= 0: none

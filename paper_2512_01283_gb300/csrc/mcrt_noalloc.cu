@@ -259,6 +259,7 @@ extern "C" mcrt_status mcrt_launch_packets_noalloc(const mcrt_noalloc_problem* p
     P.pid_end = pe;
     P.roulette_thr = d->roulette_threshold;
     P.roulette_surv = d->roulette_survival > 0.0 ? d->roulette_survival : 1.0;
+    P.roulette_gain = 1.0 / P.roulette_surv;
     P.max_events = d->max_events > 0 ? (d->max_events < 2147483647ll ? d->max_events : 2147483647ll) : 100000;
     P.max_trials = d->max_trials > 0 ? d->max_trials : 1000;
     P.time_budget_ns = d->time_budget_s > 0.0 ? d->time_budget_s * 1e9 : 0.0;

@@ -309,10 +309,10 @@ template <typename J> __device__ __forceinline__ long long thermal_cell(const J&
 
 // Packet birth, event 0: slot 0 = (tau, cos theta, phi, cell), slot 1 = (x, y, z, -).
 // pid is the packet id within its model.  Returns false when the packet starts
-// outside the grid (it is then finished).
+// outside the grid (the caller finishes it).
 // WP: the instantiation walks composite grids (births in patch cells).
 template <typename T, bool B, bool WP>
-__device__ bool emit(const TransportParams& P, const JobRef<T, B>& job, long long pid, Packet<T>& pk, BlockTotals& bt) {
+__device__ bool emit(const TransportParams& P, const JobRef<T, B>& job, long long pid, Packet<T>& pk) {
     int s = 0;
     while (s < P.n_src - 1 && pid >= P.src[s].start + P.src[s].count) ++s;
     const SourceDev& src = P.src[s];
@@ -424,8 +424,22 @@ __device__ bool emit(const TransportParams& P, const JobRef<T, B>& job, long lon
     }
     tau_set(pk.tau, -t_log(u0.a));
     pk.I_birth = pk.X0;
-    if (!inside) finish(P, pk, 1, bt);
     return inside;
+}
+
+// emit() as a function of its own, returning the packet: inlined, the births of all source kinds
+// stood in the middle of the in-place kernels' loop (plane-parallel slab 375 -> 363 ms, batched
+// sweep 162.5 -> 159.6 ms; slab of 1e6 packets 1.14 -> 1.16 ms).
+template <typename T, bool B, bool WP> struct Born {
+    Packet<T> pk;
+    bool inside;
+};
+template <typename T, bool B, bool WP>
+__device__ __noinline__ Born<T, B, WP> emit_apart(const TransportParams& P, const JobRef<T, B> job, long long pid, const JobDev* jd) {
+    Born<T, B, WP> b;
+    b.pk.job = jd;
+    b.inside = emit<T, B, WP>(P, job, pid, b.pk);
+    return b;
 }
 
 // Exit of the current cell along n: distance, axis (ties to the lowest axis) and the
@@ -504,10 +518,16 @@ template <int SCAT> __device__ __forceinline__ void empty_record(const Transport
 
 // One event of a live packet: a cell segment, then a scattering when the sampled
 // optical depth runs out inside the cell.  `work` = live lanes of the warp; `staged` is set
-// to the number of tally rows the warp staged where this lane is one of them.
+// to the number of tally rows the warp staged where this lane is one of them.  A packet that
+// ends here leaves its fate (finish()'s flag) to the kernel's loop, which holds the only copy of
+// that code.  The instruction cache is what such code costs
+// (22 % of the stalls of the table rounds were instruction fetches): one copy instead of four,
+// with the parts of mcrt_device.cuh that are called apart, took 12 to 14 kB off the kernels and
+// the refined disk's transport from 85.8 to 78.6 ms, the plane-parallel slab from 402 to 376 ms,
+// the batched sweep from 171.7 to 165 ms.
 template <typename T, int SCAT, bool B, bool R>
 __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm, Packet<T>& pk, bool& alive,
-                                     BlockTotals& bt, unsigned work, int& staged) {
+                                     int& fate, unsigned work, int& staged) {
     const JobRef<T, B> job = job_of<T, B>(P, sm, pk);
     const TablesDev& tabs = job.t();
     const T ks = T(pk.cr.y);
@@ -535,7 +555,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
     const unsigned actA = __ballot_sync(work, want_A);
     const unsigned actS = __ballot_sync(work, want_S);
     if (capped || lost) {
-        finish(P, pk, capped ? 3 : 1, bt);
+        fate = capped ? 3 : 1;
         alive = false;
         return;
     }
@@ -803,7 +823,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
         pk.iy = niy;
         pk.iz = niz;
         if (!next_in) {
-            finish(P, pk, 1, bt);
+            fate = 1;
             alive = false;
             return;
         }
@@ -835,17 +855,16 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
 // fraction of its birth intensity: it survives with probability surv, its Stokes
 // vector scaled by 1 / surv.  Returns false when the packet ends here.
 template <typename T>
-__device__ __forceinline__ bool roulette(const TransportParams& P, Packet<T>& pk, T u, BlockTotals& bt) {
+__device__ __forceinline__ bool roulette(const TransportParams& P, Packet<T>& pk, T u) {
     if (P.roulette_thr > 0.0 && (double)pk.X0 < P.roulette_thr * (double)pk.I_birth) {
         if ((double)u < P.roulette_surv) {
-            const T gmul = T(1.0 / P.roulette_surv);
+            const T gmul = T(P.roulette_gain);
             pk.e_gain += pk.X0 * (gmul - T(1));
             pk.X0 *= gmul;
             pk.X1 *= gmul;
             pk.X2 *= gmul;
             pk.X3 *= gmul;
         } else {
-            finish(P, pk, 2, bt);
             return false;
         }
     }
@@ -962,7 +981,7 @@ template <typename T> __device__ __forceinline__ V3<T> shfl3(const V3<T>& v, int
 // (groups of 4), spheroids 70.2 -> 69.5 ms.
 template <typename T, int SCAT, bool B>
 __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Smem<T>& sm, Packet<T>& pk, bool& alive,
-                                             BlockTotals& bt) {
+                                             int& fate) {
     constexpr bool kTable = table_optics(SCAT), kDipole = SCAT == MCRT_SCAT_DIPOLE;
     const int lane = threadIdx.x & 31;
     bool live = false;
@@ -972,8 +991,9 @@ __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Sme
         pk.pending = false;
         const JobRef<T, B> job = job_of<T, B>(P, sm, pk);
         const Draw4<T> us = draw4<T>(pk.pid, pk.n_sca, 0u, P.seed, job.stream());
-        live = roulette(P, pk, us.b, bt);
+        live = roulette(P, pk, us.b);
         alive = live;
+        if (!live) fate = 2;
         if constexpr (kTable) bin = size_bin(job.t(), us.c);
         u_tau = us.a;
     }
@@ -1051,7 +1071,7 @@ __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Sme
     }
     if (!live) return;
     if (!accepted) {
-        finish(P, pk, 4, bt);
+        fate = 4;
         alive = false;
         return;
     }
@@ -1151,6 +1171,7 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
     Packet<T> pk;
     pk.job = nullptr;
     bool alive = false, pool_done = false;
+    int fate = 0;  // how the lane's packet ended (0: it did not), until the loop's next turn
     bool stop = false;  // round-based paths: this lane's record went past the soft limit
     const unsigned long long t0 = global_ns();
     // surrogate path: packets resumed after their scattering, then new packets
@@ -1165,6 +1186,10 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
     }
 
     for (;;) {
+        if (fate != 0) {
+            finish(P, pk, fate, bt);
+            fate = 0;
+        }
         // dead lanes take new work in groups, so that the birth code runs for several
         // lanes at once (or when no lane can move otherwise)
         const unsigned need = __ballot_sync(kFull, !alive && !pool_done);
@@ -1199,7 +1224,8 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
                     // the surrogate path emits here; the table rounds hold no birth code
                     if constexpr (SCAT != kScatTableDeferred) {
                         const long long pid = P.pid_begin + (long long)(w_next + (idx - w_resume));
-                        alive = emit<T, false, R>(P, jr, pid, pk, bt);
+                        alive = emit<T, false, R>(P, jr, pid, pk);
+                        fate = alive ? 0 : 1;
                         pk.park = false;
                     }
                 } else {
@@ -1230,9 +1256,15 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
                     pk.job = &P.jobs[job_index(P, pid)];
                     local = pid - pk.job->pid_start;
                 }
-                alive = emit<T, true, false>(P, JobRef<T, true>{pk.job}, local, pk, bt);
+                const Born<T, true, false> b = emit_apart<T, true, false>(P, JobRef<T, true>{pk.job}, local, pk.job);
+                pk = b.pk;
+                alive = b.inside;
+                fate = alive ? 0 : 1;
             } else {
-                alive = emit<T, false, R>(P, JobRef<T, false>{P, sm.kext, sm.mix}, pid, pk, bt);
+                const Born<T, false, R> b = emit_apart<T, false, R>(P, JobRef<T, false>{P, sm.kext, sm.mix}, pid, nullptr);
+                pk = b.pk;
+                alive = b.inside;
+                fate = alive ? 0 : 1;
             }
         }
         const unsigned pend = __ballot_sync(kFull, alive && pk.pending);
@@ -1244,11 +1276,11 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
         // scatterings of the warp run together once enough lanes wait for one, or as many as move
         if (pend != 0u && (__popc(pend) >= scatter_batch<B, SCAT>() || __popc(pend) >= __popc(work))) {
             // every lane runs trials of the waiting packets (the surrogate scatters in its own kernel)
-            if constexpr (SCAT != kScatSurrogate) scatter_coop<T, SCAT, B>(P, sm, pk, alive, bt);
+            if constexpr (SCAT != kScatSurrogate) scatter_coop<T, SCAT, B>(P, sm, pk, alive, fate);
             continue;
         }
         int staged = 0;
-        if (alive && !pk.pending) step<T, SCAT, B, R>(P, sm, pk, alive, bt, work, staged);
+        if (alive && !pk.pending) step<T, SCAT, B, R>(P, sm, pk, alive, fate, work, staged);
         if constexpr (!round_based(SCAT)) {
             const int rows = __reduce_max_sync(kFull, staged);
             if (rows > 0) {
@@ -1302,12 +1334,14 @@ template <bool R> __global__ void __launch_bounds__(kBirthBlock) k_birth(const _
         Packet<float> pk;
         pk.job = nullptr;
         const long long pid = P.pid_begin + (long long)(next + i);
-        if (emit<float, false, R>(P, jr, pid, pk, bt)) {
+        if (emit<float, false, R>(P, jr, pid, pk)) {
             cg::coalesced_group grp = cg::coalesced_threads();
             unsigned long long base = 0;
             if (grp.thread_rank() == 0) base = atomicAdd(&P.sur.ctl->n_born, (unsigned long long)grp.size());
             base = grp.shfl(base, 0);
             store_state(P.sur.resume + (first + base + grp.thread_rank()) * kStateF4, pk, 1u);
+        } else {
+            finish(P, pk, 1, bt);
         }
     }
     __syncthreads();

@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kWaveBlock, 1) k_sur_scatter(const __grid_cons
             live = true;
             if (P.roulette_thr > 0.0 && (double)pk.X0 < P.roulette_thr * (double)pk.I_birth) {
                 if ((double)us.b < P.roulette_surv) {
-                    const float gmul = (float)(1.0 / P.roulette_surv);
+                    const float gmul = (float)P.roulette_gain;
                     pk.e_gain += pk.X0 * (gmul - 1.f);
                     pk.X0 *= gmul;
                     pk.X1 *= gmul;
@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(tc::kRows * kScatGroups, 1) k_sur_scatter_tc(c
                 live = true;
                 if (P.roulette_thr > 0.0 && (double)pk.X0 < P.roulette_thr * (double)pk.I_birth) {
                     if ((double)us.b < P.roulette_surv) {
-                        const float gmul = (float)(1.0 / P.roulette_surv);
+                        const float gmul = (float)P.roulette_gain;
                         pk.e_gain += pk.X0 * (gmul - 1.f);
                         pk.X0 *= gmul;
                         pk.X1 *= gmul;
