@@ -800,7 +800,8 @@ static mcrt_status launch_one(mcrt_ctx* ctx, const mcrt_launch_desc* d, mcrt_sta
     if (block % 32 != 0 || block > 128)
         return fail(ctx, MCRT_E_INVAL, "mcrt_launch_packets: block_size must be a multiple of 32, <= 128");
     const size_t smem = transport_smem_bytes(P, d->precision, block);
-    int bps = transport_max_blocks_per_sm(d->precision, P.t.model, false, block, smem, P.g.n_patches > 0);
+    int bps = transport_max_blocks_per_sm(d->precision, P.t.model, false, block, smem, P.g.n_patches > 0,
+                                          P.t.k_iso != 0);
     if (d->blocks_per_sm > 0 && d->blocks_per_sm < bps) bps = d->blocks_per_sm;
     const long long work = pe - pb;
     long long grid = (long long)ctx->n_sm * bps;
@@ -873,7 +874,8 @@ static mcrt_status launch_one(mcrt_ctx* ctx, const mcrt_launch_desc* d, mcrt_sta
             // the transport leaves room on every SM for the tally kernels of the round before
             P.sur.deferred = kScatTableDeferred;
             const size_t tsm = transport_smem_bytes(P, MCRT_FP32, 128);
-            const int bmax = transport_max_blocks_per_sm(MCRT_FP32, kScatTableDeferred, false, 128, tsm, P.g.n_patches > 0);
+            const int bmax = transport_max_blocks_per_sm(MCRT_FP32, kScatTableDeferred, false, 128, tsm, P.g.n_patches > 0,
+                                                         P.t.k_iso != 0);
             int tbps = d->blocks_per_sm > 0 ? d->blocks_per_sm : (bmax > 2 ? bmax - 2 : 1);
             if (tbps > bmax) tbps = bmax;
             const int abps = d->tally_blocks_per_sm;

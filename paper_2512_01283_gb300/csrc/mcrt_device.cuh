@@ -334,6 +334,23 @@ __device__ __forceinline__ void path_integral(T xa, T ya, T xp, T xm, const T X[
     W[3] = mad2<kSecond>(re, X[3], im, X[2]);
 }
 
+// transfer() for a2 = a3 = 0: the exponentials of the three eigenvalues are one, and what it
+// returns is the same bit for bit (an infinite depth transmits nothing).
+template <typename T>
+__device__ __forceinline__ void transfer_isotropic(const T X[4], T a, T dtau, T Y[4], T W[4], bool want_W, T wscale) {
+    const T x = t_mul(a, dtau), ea = t_exp(-x);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) Y[e] = t_mul(ea, X[e]);
+    if (want_W) {
+        const T E = t_mul(wscale, e1(x));
+        const T sp = X[0] + X[1], sm = X[0] - X[1];
+        W[0] = T(0.5) * mad2(E, sp, E, sm);
+        W[1] = T(0.5) * msb2(E, sp, E, sm);
+        W[2] = t_mul(E, X[2]);
+        W[3] = t_mul(E, X[3]);
+    }
+}
+
 // A segment's Y = e^{-M dtau} X and, with want_W, its path integral W.
 template <bool fused_xm = false, typename T>
 __device__ __forceinline__ void transfer(const T X[4], T a, T a2, T a3, T dtau, T Y[4], T W[4], bool want_W,

@@ -236,8 +236,9 @@ cudaError_t launch_transport(const TransportParams& p, int precision, int block,
 // Births of a round of the FP32 table path (k_birth): the round's new packets in the
 // waiting form after the resume list, before the round's transport launch.
 cudaError_t launch_births(const TransportParams& p, int n_sm, cudaStream_t s);
-const void* transport_kernel(int precision, int model, bool batch, bool refined = false);
-int transport_max_blocks_per_sm(int precision, int model, bool batch, int block, size_t smem, bool refined = false);
+const void* transport_kernel(int precision, int model, bool batch, bool refined = false, bool iso = false);
+int transport_max_blocks_per_sm(int precision, int model, bool batch, int block, size_t smem, bool refined = false,
+                                bool iso = false);
 size_t transport_smem_bytes(const TransportParams& p, int precision, int block);
 cudaError_t launch_image(const ImageParams& p, int precision, cudaStream_t s);
 cudaError_t launch_setup_cells(const float* ka, const float* ks, const float* bf, const float* em, long long ncell,

@@ -276,7 +276,7 @@ extern "C" mcrt_status mcrt_launch_packets_noalloc(const mcrt_noalloc_problem* p
     NA_CK(cudaGetDevice(&dev));
     NA_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const size_t smem = transport_smem_bytes(P, d->precision, block);
-    int bps = transport_max_blocks_per_sm(d->precision, P.t.model, false, block, smem);
+    int bps = transport_max_blocks_per_sm(d->precision, P.t.model, false, block, smem, false, P.t.k_iso != 0);
     if (d->blocks_per_sm > 0 && d->blocks_per_sm < bps) bps = d->blocks_per_sm;
     const long long nwork = pe - pb;
     long long grid = (long long)nsm * bps;

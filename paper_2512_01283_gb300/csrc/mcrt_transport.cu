@@ -525,7 +525,7 @@ template <int SCAT> __device__ __forceinline__ void empty_record(const Transport
 // with the parts of mcrt_device.cuh that are called apart, took 12 to 14 kB off the kernels and
 // the refined disk's transport from 85.8 to 78.6 ms, the plane-parallel slab from 402 to 376 ms,
 // the batched sweep from 171.7 to 165 ms.
-template <typename T, int SCAT, bool B, bool R>
+template <typename T, int SCAT, bool B, bool R, bool ISO>
 __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm, Packet<T>& pk, bool& alive,
                                      int& fate, unsigned work, int& staged) {
     const JobRef<T, B> job = job_of<T, B>(P, sm, pk);
@@ -626,7 +626,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
             dipole_K(dc.ca0, dc.ca1, dc.cs0, dc.cs1,
                      t_div(T(pk.cr.x), kext), t_div(ks, kext), dip_f.cos_tp, a1, a2, s11, s12);
             a3 = T(0);
-        } else if (tabs.k_iso) {
+        } else if (ISO || ((B || SCAT == kScatSurrogate) && tabs.k_iso)) {
             a1 = T(job.kext()[0].x);
             a2 = T(0);
             a3 = T(0);
@@ -639,10 +639,14 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
         const T a = a1 - omega;
         const T dtau = kext * ell;
         T Xg[4] = {pk.X0, pk.X1, pk.X2, pk.X3};
-        rotate_qu<SCAT == MCRT_SCAT_DIPOLE ? kSecond : kFirst>(Xg[1], Xg[2], c2, s2);
+        if constexpr (!ISO) rotate_qu<SCAT == MCRT_SCAT_DIPOLE ? kSecond : kFirst>(Xg[1], Xg[2], c2, s2);
         T Yg[4], Wg[4];
-        transfer<SCAT == kScatTableDeferred>(Xg, a, a2, a3, dtau, Yg, Wg, want_S || SCAT == MCRT_SCAT_DIPOLE, ell);
-        rotate_back(Yg[1], Yg[2], c2, s2);
+        if constexpr (ISO) {
+            transfer_isotropic(Xg, a, dtau, Yg, Wg, want_S, ell);
+        } else {
+            transfer<SCAT == kScatTableDeferred>(Xg, a, a2, a3, dtau, Yg, Wg, want_S || SCAT == MCRT_SCAT_DIPOLE, ell);
+            rotate_back(Yg[1], Yg[2], c2, s2);
+        }
         // absorbed energy, one FP64 atomic per same-cell group
         {
             const unsigned gmax = kGroups ? __reduce_max_sync(actA, (unsigned)__popc(group)) : 1u;
@@ -666,7 +670,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
                 // consecutive slots; a warp that would run past the queue's end writes
                 // empty records and tallies in place below
                 T Wl1 = Wg[1], Wl2 = Wg[2];  // path integral in the packet's basis
-                rotate_back(Wl1, Wl2, c2, s2);
+                if constexpr (!ISO) rotate_back(Wl1, Wl2, c2, s2);
                 const int lead = __ffs(actS) - 1;
                 const unsigned cnt = (unsigned)__popc(actS);
                 unsigned long long base = 0;
@@ -738,7 +742,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
         // the table rounds keep no in-place tally (smaller kernel): a segment that finds
         // no queue space is counted and fails the launch, which the soft limit rules out
         if (SCAT != kScatTableDeferred && want_S && !queued) {
-            rotate_back(Wg[1], Wg[2], c2, s2);
+            if constexpr (!ISO) rotate_back(Wg[1], Wg[2], c2, s2);
             const unsigned gmax = kGroups ? __reduce_max_sync(actS, (unsigned)__popc(group)) : 1u;
             pk.n_tally++;
             double* Sc = job.S() + (size_t)c32 * (size_t)P.n_cam * 4;
@@ -1138,7 +1142,11 @@ constexpr int min_blocks() {
     return sizeof(T) != 4 ? 1 : (SCAT == kScatTableDeferred ? MCRT_ROUND_MIN_BLOCKS : MCRT_MIN_BLOCKS);
 }
 
-template <typename T, int SCAT, bool B, bool R>
+// ISO: the extinction does not depend on direction or polarization (spherical grains), so that a
+// segment needs one exponential for the three eigenvalues and neither the grain frame nor the
+// extinction table: sphere of 1e5 packets 0.58 -> 0.49 ms; kernels apart, because as a branch
+// the extra code cost the others 2 to 6 %.  The jobs of a batched launch may differ in it.
+template <typename T, int SCAT, bool B, bool R, bool ISO>
 __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
     k_transport(const __grid_constant__ TransportParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1280,7 +1288,7 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
             continue;
         }
         int staged = 0;
-        if (alive && !pk.pending) step<T, SCAT, B, R>(P, sm, pk, alive, fate, work, staged);
+        if (alive && !pk.pending) step<T, SCAT, B, R, ISO>(P, sm, pk, alive, fate, work, staged);
         if constexpr (!round_based(SCAT)) {
             const int rows = __reduce_max_sync(kFull, staged);
             if (rows > 0) {
@@ -1380,35 +1388,39 @@ size_t transport_smem_bytes(const TransportParams& p, int precision, int block) 
     return kx + mix + cams + stage;
 }
 
-template <typename T, int SCAT, bool B> const void* kernel_of(bool refined) {
+template <typename T, int SCAT, bool B, bool ISO> const void* kernel_of(bool refined) {
     if constexpr (walks_patches(SCAT, B))
-        if (refined) return (const void*)k_transport<T, SCAT, B, true>;
-    return (const void*)k_transport<T, SCAT, B, false>;
+        if (refined) return (const void*)k_transport<T, SCAT, B, true, ISO>;
+    return (const void*)k_transport<T, SCAT, B, false, ISO>;
+}
+template <typename T, int SCAT> const void* kernel_of(bool refined, bool iso) {
+    return iso ? kernel_of<T, SCAT, false, true>(refined) : kernel_of<T, SCAT, false, false>(refined);
 }
 
-template <typename T> const void* kernel_of_model(int model, bool batch, bool refined) {
+template <typename T> const void* kernel_of_model(int model, bool batch, bool refined, bool iso) {
     if (model == MCRT_SCAT_DIPOLE)  // single-model launches only
-        return kernel_of<T, MCRT_SCAT_DIPOLE, false>(refined);
+        return kernel_of<T, MCRT_SCAT_DIPOLE, false, false>(refined);
+    // the jobs of a batched launch may differ in their extinction
     if (model == MCRT_SCAT_TABLE)
-        return batch ? kernel_of<T, MCRT_SCAT_TABLE, true>(false) : kernel_of<T, MCRT_SCAT_TABLE, false>(refined);
-    return batch ? kernel_of<T, MCRT_SCAT_RAYLEIGH, true>(false) : kernel_of<T, MCRT_SCAT_RAYLEIGH, false>(refined);
+        return batch ? kernel_of<T, MCRT_SCAT_TABLE, true, false>(false) : kernel_of<T, MCRT_SCAT_TABLE>(refined, iso);
+    return batch ? kernel_of<T, MCRT_SCAT_RAYLEIGH, true, false>(false)
+                 : kernel_of<T, MCRT_SCAT_RAYLEIGH>(refined, iso);
 }
 
-const void* transport_kernel(int precision, int model, bool batch, bool refined) {
-    return precision == MCRT_FP64 ? kernel_of_model<double>(model, batch, refined)
-                                  : kernel_of_model<float>(model, batch, refined);
+const void* transport_kernel(int precision, int model, bool batch, bool refined, bool iso) {
+    return precision == MCRT_FP64 ? kernel_of_model<double>(model, batch, refined, iso)
+                                  : kernel_of_model<float>(model, batch, refined, iso);
 }
 
-const void* transport_kernel_rounds(int model, bool refined) {
-    if (model == kScatSurrogate) return (const void*)k_transport<float, kScatSurrogate, false, false>;
-    return refined ? (const void*)k_transport<float, kScatTableDeferred, false, true>
-                   : (const void*)k_transport<float, kScatTableDeferred, false, false>;
+const void* transport_kernel_rounds(int model, bool refined, bool iso) {
+    if (model == kScatSurrogate) return (const void*)k_transport<float, kScatSurrogate, false, false, false>;
+    return kernel_of<float, kScatTableDeferred>(refined, iso);
 }
 
-int transport_max_blocks_per_sm(int precision, int model, bool batch, int block, size_t smem, bool refined) {
+int transport_max_blocks_per_sm(int precision, int model, bool batch, int block, size_t smem, bool refined, bool iso) {
     int nb = 0;
-    const void* k = round_based(model) ? transport_kernel_rounds(model, refined)
-                                        : transport_kernel(precision, model, batch, refined);
+    const void* k = round_based(model) ? transport_kernel_rounds(model, refined, iso)
+                                        : transport_kernel(precision, model, batch, refined, iso);
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, block, smem) != cudaSuccess) return 1;
     return nb > 0 ? nb : 1;
@@ -1416,8 +1428,9 @@ int transport_max_blocks_per_sm(int precision, int model, bool batch, int block,
 
 cudaError_t launch_transport(const TransportParams& p, int precision, int block, int grid, cudaStream_t s) {
     const size_t smem = transport_smem_bytes(p, precision, block);
-    const void* k = p.sur.deferred ? transport_kernel_rounds(p.sur.deferred, p.g.n_patches > 0)
-                                   : transport_kernel(precision, p.t.model, p.jobs != nullptr, p.g.n_patches > 0);
+    const void* k = p.sur.deferred ? transport_kernel_rounds(p.sur.deferred, p.g.n_patches > 0, p.t.k_iso != 0)
+                                   : transport_kernel(precision, p.t.model, p.jobs != nullptr, p.g.n_patches > 0,
+                                                      p.t.k_iso != 0);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
