@@ -722,8 +722,9 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
                     } else {
                         float4* r = P.sur.records + idx * kTableRecordF4;
                         if (queued) {
-                            r[0] = make_float4((float)n.x, (float)n.y, (float)n.z, (float)Wg[0]);
-                            r[1] = make_float4((float)Wl1, (float)Wl2, (float)Wg[3], __uint_as_float(c32));
+                            // streamed: the tally reads them once, the L2 is the cells'
+                            __stcs(r, make_float4((float)n.x, (float)n.y, (float)n.z, (float)Wg[0]));
+                            __stcs(r + 1, make_float4((float)Wl1, (float)Wl2, (float)Wg[3], __uint_as_float(c32)));
                         } else {
                             r[1] = make_float4(0.f, 0.f, 0.f, __uint_as_float(0xffffffffu));
                         }
@@ -1133,9 +1134,10 @@ __device__ __forceinline__ int job_index(const TransportParams& P, long long gpi
 }
 
 // resident blocks per SM of the table-round instantiation: without the camera loop
-// and its staging slots it fits more warps per SM
+// and its staging slots it fits more warps per SM.  6 (80 registers, almost no spills) against 7
+// and 8, ms: 1e7 star packets of the 192^3 disk 38.5, 39.4, 41; refined disk 73.7, 74.3, 89
 #ifndef MCRT_ROUND_MIN_BLOCKS
-#define MCRT_ROUND_MIN_BLOCKS 7
+#define MCRT_ROUND_MIN_BLOCKS 6
 #endif
 template <typename T, int SCAT>
 constexpr int min_blocks() {
@@ -1213,7 +1215,6 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
                 // the record queue is near its end: work items taken now wait for the
                 // next round without a segment
                 const bool full = *reinterpret_cast<volatile unsigned long long*>(&P.sur.ctl->full) != 0ull;
-                pk.park = false;
                 const JobRef<T, false> jr{P, sm.kext, sm.mix};
                 if (idx < w_resume) {
                     if constexpr (sizeof(T) == 4) {
@@ -1239,7 +1240,7 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
                 } else {
                     pool_done = true;
                 }
-                if (alive && (full || stop)) park_packet(P, pk, alive);
+                pk.park = alive && (full || stop);
             }
             if (alive && pk.park && !pk.pending) {  // before the next segment, outside collective steps
                 stop = true;
