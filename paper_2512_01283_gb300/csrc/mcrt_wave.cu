@@ -903,8 +903,12 @@ __global__ void __launch_bounds__(tc::kRows * kScatGroups, 1) k_sur_scatter_tc(c
 // a row of its own and issues one contiguous FP64 bulk reduction into S[cell]; lanes
 // share nothing, so no lane waits for another.  Same arithmetic as the in-place tally
 // of k_transport (table_matrix, plane_rotation, apply_plane).
-constexpr int kTabBlock = 128;
-constexpr int kTabSlots = 2;  // staging rows per lane (1 or 2), alternated from tile to tile
+// One staging row per lane: a second one, alternated from tile to tile, lets the reduction of the
+// tile before drain, but halves the warps that fit (8 cameras: 24 warps per SM against 12).  ms
+// with two rows and blocks of 128, with one and 128, with one and 256 and the records streamed
+// past the L2: 64^3 disk 2.20, 2.12, 2.09; refined disk 53.8, 53.1, 52.0; 192^3 disk, 1e7 packets,
+// 60.0, 58.4, 57.6.  Blocks of 64 and fewer of them per SM were slower.
+constexpr int kTabBlock = 256;
 // a lane's staging row: the cameras' rows, padded by 16 B so that the 16-byte stores of
 // a quarter-warp's lanes (rows 8 c + 4 words apart) fall in different bank groups
 __host__ __device__ constexpr int tab_row_bytes(int ncam) { return ncam * 32 + 16; }
@@ -925,22 +929,19 @@ __global__ void __launch_bounds__(kTabBlock) k_tab_tally(const __grid_constant__
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     const int ncam = P.n_cam;
     const int row = tab_row_bytes(ncam);
-    // row of (warp, slot, lane) at index (warp * kTabSlots + slot) * 32 + lane
-    unsigned char* const rows = s_stage + ((size_t)(threadIdx.x >> 5) * kTabSlots * 32 + lane) * row;
+    unsigned char* const dst = s_stage + (size_t)threadIdx.x * row;
     const unsigned long long nreq = P.sur.ctl->n_rec[P.sur.rec_slot];
     const unsigned long long nrec = nreq < P.sur.rec_cap ? nreq : P.sur.rec_cap;
     const unsigned long long ntile = (nrec + 31) / 32;
     const unsigned long long stride = (unsigned long long)gridDim.x * wpb;
-    // the next tile's record is loaded while this one is converted; a lane's two rows
-    // alternate, so that a row is rewritten only once the reduction issued from it two
-    // tiles before has read it (every lane commits one bulk group per tile, empty when
-    // it issues none, so "all but the newest group" is that reduction)
+    // the next tile's record is loaded while this one is converted; the lane's row is rewritten
+    // once the reduction issued from it has read it
     auto load = [&](unsigned long long t, float4& a, float4& b) {
         const unsigned long long rec = t * 32 + (unsigned)lane;
         if (t < ntile && rec < nrec) {
             const float4* r = P.sur.records + rec * kTableRecordF4;
-            a = r[0];
-            b = r[1];
+            a = __ldcs(r);
+            b = __ldcs(r + 1);
         } else {
             b.w = __uint_as_float(0xffffffffu);
         }
@@ -948,16 +949,12 @@ __global__ void __launch_bounds__(kTabBlock) k_tab_tally(const __grid_constant__
     float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
     unsigned long long tile = (unsigned long long)blockIdx.x * wpb + (threadIdx.x >> 5);
     load(tile, n0, n1);
-    for (unsigned it = 0; tile < ntile; ++it, tile += stride) {
+    for (; tile < ntile; tile += stride) {
         const float4 r0 = n0, r1 = n1;
         load(tile + stride, n0, n1);
         const unsigned cell = __float_as_uint(r1.w);
         if (cell != 0xffffffffu) {
-            unsigned char* const dst = rows + (size_t)(it % kTabSlots) * 32 * row;
-            if constexpr (kTabSlots == 1)
-                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            else
-                asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             const V3<float> n{r0.x, r0.y, r0.z};
             const float W[4] = {r0.w, r1.x, r1.y, r1.z};
             V3<float> th, ph;
@@ -990,7 +987,7 @@ __global__ void __launch_bounds__(kTabBlock) k_tab_tally(const __grid_constant__
 
 size_t tab_tally_smem(const TransportParams& p) {
     return (size_t)2 * p.t.n_theta * sizeof(float4) + 12 * kMaxCams * sizeof(float) +
-           (size_t)(kTabBlock / 32) * kTabSlots * 32 * (size_t)tab_row_bytes(p.n_cam > 0 ? p.n_cam : 1);
+           (size_t)kTabBlock * (size_t)tab_row_bytes(p.n_cam > 0 ? p.n_cam : 1);
 }
 
 }  // namespace
