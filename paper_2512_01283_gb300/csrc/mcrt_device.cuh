@@ -430,9 +430,13 @@ __device__ __forceinline__ PlaneRot<T> plane_rotation(const V3<T>& n, const V3<T
         B2 = dot<F>(ph, th2);
     }
     PlaneRot<T> r;
-    // both pairs have the length sin(Theta) >= 1e-6, or that of phi(n) across n2
-    double_angle<F, false>(A1, B1, r.c1, r.s1);
-    double_angle<F, false>(A2, B2, r.c2, r.s2);
+    // Both pairs have the length sin(Theta) >= 1e-6, or that of phi(n) across n2, so that none is
+    // tiny.  FP64 keeps the test all the same: the branches separate its long dependent chains for
+    // the compiler, whose schedule without them ran 4 to 8 % slower (24^3 disk of 1e5 packets 10.9
+    // against 10.5 ms, 40^3 of 5e4 12.9 against 11.8).
+    constexpr bool kTest = sizeof(T) == 8;
+    double_angle<F, kTest>(A1, B1, r.c1, r.s1);
+    double_angle<F, kTest>(A2, B2, r.c2, r.s2);
     return r;
 }
 
@@ -442,7 +446,7 @@ __device__ __forceinline__ T plane_Q(const V3<T>& th, const V3<T>& ph, const V3<
     const T A1 = dot(n2, th), B1 = dot(n2, ph);
     if (mad2(A1, A1, B1, B1) < T(1e-12)) return X[1];
     T c1, s1;
-    double_angle<kFirst, false>(A1, B1, c1, s1);
+    double_angle<kFirst, sizeof(T) == 8>(A1, B1, c1, s1);  // as in plane_rotation
     return mad2(c1, X[1], s1, X[2]);
 }
 
