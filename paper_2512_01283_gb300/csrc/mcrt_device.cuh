@@ -258,12 +258,21 @@ template <typename T> __device__ __noinline__ Pair<T> sincos_apart(T y) {
     return p;
 }
 
+// With `calls` false inlined, for the surrogate's transport, where every segment needs it (64^3 disk,
+// 42 rounds: 7.50 -> 7.32 ms).
+template <bool calls, typename T> __device__ __forceinline__ Pair<T> sincos_of(T y) {
+    if constexpr (calls) return sincos_apart(y);
+    Pair<T> p;
+    t_sincos(y, &p.a, &p.b);
+    return p;
+}
+
 // int_0^1 e^{-(x - i y) s} ds = (a, b) for y != 0
-template <typename T> __device__ __forceinline__ Pair<T> e1_turning(T x, T y) {
+template <bool calls, typename T> __device__ __forceinline__ Pair<T> e1_turning(T x, T y) {
     if (fabs(x) + fabs(y) < T(1e-4))
         return Pair<T>{t_fma(msb2(x, x, y, y), T(1.0 / 6.0), t_fma(-x, T(0.5), T(1))),
                        msb2(y, T(0.5), t_mul(x, y), T(1.0 / 3.0))};
-    const Pair<T> half = sincos_apart(T(0.5) * y);
+    const Pair<T> half = sincos_of<calls>(T(0.5) * y);
     const T sh = half.a, sy = T(2) * sh * half.b;
     const T ex = t_exp(-x);
     const T nr = t_fma(T(2) * ex * sh, sh, -t_expm1(-x));  // 1 - e^{-x} cos y
@@ -276,9 +285,9 @@ template <typename T> __device__ __forceinline__ Pair<T> e1_turning(T x, T y) {
 // slab 347.7 instead of 352.2 (a slab that does turn them, 1e6 packets, 20.2 instead of 19.9).  The
 // table rounds are faster with it inlined (refined disk's transport 78.6 against 79.8 ms), as are
 // the surrogate's, whose media all turn (7.6 against 7.8 ms).
-template <typename T> __device__ __noinline__ Pair<T> e1_turning_apart(T x, T y) { return e1_turning(x, y); }
+template <typename T> __device__ __noinline__ Pair<T> e1_turning_apart(T x, T y) { return e1_turning<true>(x, y); }
 
-template <bool apart, typename T> __device__ __forceinline__ void e1_complex(T x, T y, T& re, T& im) {
+template <bool apart, bool calls, typename T> __device__ __forceinline__ void e1_complex(T x, T y, T& re, T& im) {
     if (y == T(0)) {
         re = e1(x);
         im = T(0);
@@ -288,7 +297,7 @@ template <bool apart, typename T> __device__ __forceinline__ void e1_complex(T x
     if constexpr (apart)
         p = e1_turning_apart(x, y);
     else
-        p = e1_turning(x, y);
+        p = e1_turning<calls>(x, y);
     re = p.a;
     im = p.b;
 }
@@ -301,7 +310,7 @@ template <typename T> struct Decay {
     bool thick;
 };
 
-template <typename T> __device__ __forceinline__ Decay<T> decay_of(T xa, T xb, T ya, T xp, T xm) {
+template <bool calls = true, typename T> __device__ __forceinline__ Decay<T> decay_of(T xa, T xb, T ya, T xp, T xm) {
     Decay<T> d;
     d.ea = t_exp(-xa);
     d.thick = !(fabs(xb) <= T(10));
@@ -317,7 +326,7 @@ template <typename T> __device__ __forceinline__ Decay<T> decay_of(T xa, T xb, T
     d.s3 = T(0);
     d.c3 = T(1);
     if (ya != T(0)) {
-        const Pair<T> p = sincos_apart(ya);
+        const Pair<T> p = sincos_of<calls>(ya);
         d.s3 = p.a;
         d.c3 = p.b;
     }
@@ -340,14 +349,14 @@ template <typename T> __device__ __forceinline__ void apply_decay(const Decay<T>
 
 // W = wscale * int_0^1 e^{-M dtau s} ds X (wscale = dtau gives the optical-depth integral,
 // wscale = ell the path-length one, which needs no division by kappa_ext)
-template <bool apart, typename T>
+template <bool apart, bool calls, typename T>
 __device__ __forceinline__ void path_integral(T xa, T ya, T xp, T xm, const T X[4], T W[4], T wscale) {
     const T sp = X[0] + X[1], sm = X[0] - X[1];
     const T Ep = t_mul(wscale, e1(xp)), Em = t_mul(wscale, e1(xm));
     W[0] = T(0.5) * mad2(Ep, sp, Em, sm);
     W[1] = T(0.5) * msb2(Ep, sp, Em, sm);
     T re, im;
-    e1_complex<apart>(xa, ya, re, im);
+    e1_complex<apart, calls>(xa, ya, re, im);
     re = t_mul(re, wscale);
     im = t_mul(im, wscale);
     W[2] = msb2(re, X[2], im, X[3]);
@@ -372,13 +381,13 @@ __device__ __forceinline__ void transfer_isotropic(const T X[4], T a, T dtau, T 
 }
 
 // A segment's Y = e^{-M dtau} X and, with want_W, its path integral W.
-template <bool fused_xm = false, bool apart = false, typename T>
+template <bool fused_xm = false, bool apart = false, bool calls = true, typename T>
 __device__ __forceinline__ void transfer(const T X[4], T a, T a2, T a3, T dtau, T Y[4], T W[4], bool want_W,
                                          T wscale) {
     const T xa = t_mul(a, dtau), xb = t_mul(a2, dtau), ya = t_mul(a3, dtau);
     const T xp = t_fma(a2, dtau, xa), xm = fused_xm ? t_fma(a, dtau, -xb) : t_add(xa, -xb);
-    apply_decay(decay_of(xa, xb, ya, xp, xm), X, Y);
-    if (want_W) path_integral<apart>(xa, ya, xp, xm, X, W, wscale);
+    apply_decay(decay_of<calls>(xa, xb, ya, xp, xm), X, Y);
+    if (want_W) path_integral<apart, calls>(xa, ya, xp, xm, X, W, wscale);
 }
 
 // Full App. A cell step with source S (per unit dtau) and the extinction matrix K:
@@ -392,7 +401,7 @@ template <typename T> __device__ __forceinline__ CellStep<T> cell_coeffs(T a1, T
     const T xm = t_add(xa, -xb);
     CellStep<T> c;
     c.d = decay_of(xa, xb, ya, t_fma(a2, dtau, xa), xm);
-    path_integral<false>(xa, ya, t_add(xa, xb), xm, S, c.W, dtau);
+    path_integral<false, true>(xa, ya, t_add(xa, xb), xm, S, c.W, dtau);
     return c;
 }
 template <typename T> __device__ __forceinline__ void cell_step(const CellStep<T>& c, T X[4]) {

@@ -644,7 +644,8 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
         if constexpr (ISO) {
             transfer_isotropic(Xg, a, dtau, Yg, Wg, want_S, ell);
         } else {
-            transfer<SCAT == kScatTableDeferred, !round_based(SCAT)>(Xg, a, a2, a3, dtau, Yg, Wg, want_S || SCAT == MCRT_SCAT_DIPOLE, ell);
+            transfer<SCAT == kScatTableDeferred, !round_based(SCAT), SCAT != kScatSurrogate>(
+                Xg, a, a2, a3, dtau, Yg, Wg, want_S || SCAT == MCRT_SCAT_DIPOLE, ell);
             rotate_back(Yg[1], Yg[2], c2, s2);
         }
         // absorbed energy, one FP64 atomic per same-cell group
