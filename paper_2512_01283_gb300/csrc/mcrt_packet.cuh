@@ -65,7 +65,9 @@ __device__ __forceinline__ void red_add(double* p, double v) {
 // rows + r * stride) are added to the places at(r) (nullptr: none), consecutive lanes
 // taking consecutive values, so that a row is one or a few coalesced reductions.  The values
 // are staged in the arithmetic type and widened here, every other one on the FP64 pipe and
-// the others with integer operations, which balances the two.
+// the others with integer operations, which balances the two.  The warp barriers order the
+// rows and places, which other lanes staged, before their reads here, and these reads before
+// the next rows; neither a ballot nor a warp reduction does.
 //
 // The in-place kernels issue instructions, not bytes (65 to 69 % of the issue slots, 0.03 % of
 // DRAM on the plane-parallel slab).  A bulk reduction per lane has uniform operands, so the
@@ -77,6 +79,7 @@ __device__ __forceinline__ void red_add(double* p, double v) {
 // 1.08e10 rows/s against 1.03e10 at spread positions).
 template <typename T, typename At>
 __device__ __forceinline__ void reduce_rows(int n, int lane, const T* rows, int stride, int nv, At at) {
+    __syncwarp();
     int rec = lane / nv, val = lane - rec * nv;
     const int dr = 32 / nv, dv = 32 - dr * nv;
     bool pipe = false;
@@ -92,6 +95,7 @@ __device__ __forceinline__ void reduce_rows(int n, int lane, const T* rows, int 
             rec++;
         }
     }
+    __syncwarp();
 }
 
 // alpha1..3 at cos(theta'), linear in theta' on the table grid

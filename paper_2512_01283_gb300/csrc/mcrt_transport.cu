@@ -1298,7 +1298,6 @@ __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))
                 const T* const r = reinterpret_cast<const T*>(s_stage);
                 double* const* const at = reinterpret_cast<double* const*>(r + 32 * stride);
                 reduce_rows(rows, threadIdx.x & 31, r, stride, 4 * P.n_cam, [&](int k) { return at[k]; });
-                __syncwarp();
             }
         }
     }
