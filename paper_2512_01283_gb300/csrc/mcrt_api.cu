@@ -859,8 +859,8 @@ static mcrt_status launch_one(mcrt_ctx* ctx, const mcrt_launch_desc* d, mcrt_sta
         P.sur.env_margin = validate ? 0.f : 0.05f;
         P.sur.ctl = ctx->d_wave;
         P.sur.records = ctx->d_records;
-        P.sur.rec_cap = ctx->rec_cap;
-        P.sur.rec_soft = ctx->rec_cap - margin;
+        P.sur.rec_cap = MCRT_REC_LIMIT > 0 ? (unsigned long long)MCRT_REC_LIMIT : ctx->rec_cap;
+        P.sur.rec_soft = MCRT_REC_LIMIT > 0 ? P.sur.rec_cap : ctx->rec_cap - margin;
         P.sur.suspend = ctx->d_susp;
         P.sur.resume = ctx->d_res;
         int n_rounds = 0;

@@ -24,6 +24,11 @@ constexpr int kMaxPatches = 64;
 #ifndef MCRT_TABLE_ROUND_RECORDS
 #define MCRT_TABLE_ROUND_RECORDS 32
 #endif
+// > 0: only this many slots of the record queue, and none held back, so that it runs over
+// (builds that test what then happens).
+#ifndef MCRT_REC_LIMIT
+#define MCRT_REC_LIMIT 0
+#endif
 constexpr int kMaxCams = MCRT_MAX_CAMERAS;
 constexpr int kMaxSources = MCRT_MAX_SOURCES;
 // scattering-model id of the transport instantiation that defers the optics to the

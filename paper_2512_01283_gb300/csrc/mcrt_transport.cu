@@ -516,6 +516,26 @@ template <int SCAT> __device__ __forceinline__ void empty_record(const Transport
         P.sur.records[k * kTableRecordF4 + 1] = make_float4(0.f, 0.f, 0.f, __uint_as_float(0xffffffffu));
 }
 
+// Source tally of one segment by its lane alone, from the mixture's table: what the network path
+// does for a segment without a place in the queue.  A function of its own, since it hardly ever runs.
+template <typename T> struct Stokes {
+    T v[4];
+};
+template <typename T>
+__device__ __noinline__ void tally_apart(const TransportParams& P, const T* cams, const float4* mix, unsigned cell,
+                                         const V3<T> n, const V3<T> th, const V3<T> ph, const Stokes<T> W) {
+    double* const Sc = P.S + (size_t)cell * (size_t)P.n_cam * 4;
+    for (int k = 0; k < P.n_cam; ++k) {
+        V3<T> Om, thc, phc;
+        load_camera(cams + 12 * k, Om, thc, phc);
+        T Pm[6], sv[4];
+        table_matrix(mix, P.t.n_theta, dot(n, Om), Pm);
+        apply_plane(plane_rotation(n, th, ph, Om, thc, phc), Pm, W.v, sv);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) red_add(Sc + 4 * k + e, widen(sv[e]));
+    }
+}
+
 // One event of a live packet: a cell segment, then a scattering when the sampled
 // optical depth runs out inside the cell.  `work` = live lanes of the warp; `staged` is set
 // to the number of tally rows the warp staged where this lane is one of them.  A packet that
@@ -669,7 +689,7 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
                 // the segment's tally waits for its own kernel: one record per lane (64 B
                 // with the network's inputs, 32 B for the tables), the warp's records in
                 // consecutive slots; a warp that would run past the queue's end writes
-                // empty records and tallies in place below
+                // empty records
                 T Wl1 = Wg[1], Wl2 = Wg[2];  // path integral in the packet's basis
                 if constexpr (!ISO) rotate_back(Wl1, Wl2, c2, s2);
                 const int lead = __ffs(actS) - 1;
@@ -734,16 +754,23 @@ __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm
                 }
                 // a lane whose record lands past the soft limit parks its packet before its
                 // next segment and parks all work it takes afterwards, so each thread adds
-                // at most one record beyond it and the queue cannot run over (the in-place
-                // tally below is a guard that stays unused)
+                // at most one record beyond it and the queue cannot run over
                 if (idx >= P.sur.rec_soft) pk.park = true;
                 if (lane == lead && last >= P.sur.rec_soft) atomicExch(&P.sur.ctl->full, 1ull);
                 if (!queued && lane == lead) atomicAdd(&P.sur.ctl->cnt[kCntOverflow], (unsigned long long)cnt);
             }
         }
-        // the table rounds keep no in-place tally (smaller kernel): a segment that finds
-        // no queue space is counted and fails the launch, which the soft limit rules out
-        if (SCAT != kScatTableDeferred && want_S && !queued) {
+        // a segment that finds no queue space, which the soft limit rules out: the network path
+        // tallies it with the tables at once; the table rounds hold no such code, it is counted
+        // and the launch fails
+        if constexpr (SCAT == kScatSurrogate) {
+            if (want_S && !queued) {
+                if constexpr (!ISO) rotate_back(Wg[1], Wg[2], c2, s2);
+                pk.n_tally++;
+                tally_apart(P, sm.cam, sm.mix, c32, n, th, ph, Stokes<T>{{Wg[0], Wg[1], Wg[2], Wg[3]}});
+            }
+        }
+        if (!round_based(SCAT) && want_S) {
             if constexpr (!ISO) rotate_back(Wg[1], Wg[2], c2, s2);
             const unsigned gmax = kGroups ? __reduce_max_sync(actS, (unsigned)__popc(group)) : 1u;
             pk.n_tally++;
@@ -1382,8 +1409,8 @@ size_t transport_smem_bytes(const TransportParams& p, int precision, int block) 
     const size_t kx = batch ? 0 : (size_t)p.t.n_ktheta * sizeof(float4);
     const size_t mix = (!batch && p.t.model == MCRT_SCAT_TABLE) ? 2 * (size_t)p.t.n_theta * sizeof(float4) : 0;
     const size_t cams = 12 * (size_t)p.n_cam * tsize;
-    // the table rounds tally in their own kernel: no staging slots
-    const size_t stage = p.sur.deferred == kScatTableDeferred || p.n_cam == 0
+    // the round-based paths tally in a kernel of their own: no staged rows
+    const size_t stage = p.sur.deferred != 0 || p.n_cam == 0
                              ? 0
                              : (size_t)(block / 32) * stage_warp_bytes(p.n_cam, (int)tsize);
     return kx + mix + cams + stage;
