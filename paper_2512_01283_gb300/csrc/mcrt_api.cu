@@ -23,8 +23,8 @@ struct mcrt_ctx {
     cudaStream_t stream = nullptr;
     int device = 0;
     int n_sm = 0;
-    float4* d_cells = nullptr;      // one allocation: cells, work area, patches
-    PatchDev* d_patches = nullptr;  // static mesh refinement
+    float4* d_cells = nullptr;
+    PatchDev* d_patches = nullptr;  // static mesh refinement: behind d_work, in its allocation
     bool has_emissivity = false;
     // optics: one allocation, that of d_kext
     bool tables_set = false;
@@ -282,13 +282,11 @@ static mcrt_status create_grid(const char* me, mcrt_ctx** out, int32_t nx, int32
     c->has_emissivity = emissivity != nullptr;
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device);
-    const size_t cell_bytes = round256((size_t)ncell * 2 * sizeof(float4));
-    if (e == cudaSuccess)
-        e = cudaMalloc(&c->d_cells, cell_bytes + round256(kWorkBytes) + hp.size() * sizeof(PatchDev));
-    if (e == cudaSuccess) {
-        c->d_work = reinterpret_cast<unsigned char*>(c->d_cells) + cell_bytes;
-        if (n_patches > 0) c->d_patches = reinterpret_cast<PatchDev*>(c->d_work + round256(kWorkBytes));
-    }
+    // The cells alone: records that fill whole 2 MB pages (64^3, 128^3) would take one page more
+    // with the small work area behind them, and a creation 10 % longer (128^3: 736 us against 670).
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_cells, (size_t)ncell * 2 * sizeof(float4));
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_work, round256(kWorkBytes) + hp.size() * sizeof(PatchDev));
+    if (e == cudaSuccess && n_patches > 0) c->d_patches = reinterpret_cast<PatchDev*>(c->d_work + round256(kWorkBytes));
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
     if (e != cudaSuccess) {
@@ -1082,6 +1080,7 @@ mcrt_status mcrt_destroy(mcrt_ctx* ctx) {
     if (!ctx) return MCRT_OK;
     free_tables(ctx);
     cudaFree(ctx->d_cells);
+    cudaFree(ctx->d_work);
     cudaFree(ctx->d_cdf);
     cudaFree(ctx->d_S);
     cudaFree(ctx->d_absorbed);
