@@ -168,13 +168,14 @@ __global__ void k_labels(LabelTables T, int n, const float* __restrict__ in, flo
 // A block takes tiles of 16 MT rows through all layers: weights (119 kB) and activations in
 // shared memory, the pre-activations in the registers of the warp that owns their 16 columns,
 // which also owns them on the way back.  A layer's gradient overwrites its activations.  The
-// weight gradients of a tile are added to the result with FP32 reductions of two columns.
+// weight gradients of a tile are added with FP32 reductions of two columns to one of n_parts
+// partial gradients, which the blocks share by index; folded() sums these in FP64.
 //
 // What bounds it: at a tile per SM the chain of ten small products (22 us for 2048 rows), at many
 // tiles the shared-memory reads of the operands (216 us for 65536 rows).  A gradient call, host
 // arrays to host arrays, against one launch per product and epilogue with every operand through
-// memory (25 dependent launches): 2048 rows 88 us (400), 8192 119 us (552), 2^20 3.8 ms (53.9);
-// a training step of 1024 rows 45 us (284), of 8192 70 us (439).
+// memory (25 dependent launches): 2048 rows 82 us (395), 8192 102 us (545), 2^20 3.9 ms (54.1);
+// a training step of 1024 rows 45 us (278), of 8192 66 us (436).
 // ---------------------------------------------------------------------------------
 __device__ __forceinline__ float silu_f(float z) { return mlp::silu(z); }
 __device__ __forceinline__ float silu_grad_f(float z) { return mlp::silu_grad(z); }
@@ -211,7 +212,7 @@ __device__ __forceinline__ void ldsm_x4_t(unsigned a, unsigned& r0, unsigned& r1
 template <int MT>
 __global__ void __launch_bounds__(kPassThreads, 1)
     k_pass(int B, const float* __restrict__ in, const float* __restrict__ target, const LossWeights lw,
-           const bf16* __restrict__ wbf, const float* __restrict__ params, float* __restrict__ grads,
+           const bf16* __restrict__ wbf, const float* __restrict__ params, float* __restrict__ parts, int n_parts,
            double* __restrict__ loss, const unsigned* __restrict__ iter) {
     constexpr int R = 16 * MT;
     extern __shared__ __align__(16) unsigned char pass_sm[];
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(kPassThreads, 1)
     bf16* const hs = xs + R * kLdX;
     bf16* const ys = hs + 4 * R * kLdH;
     double* const part = reinterpret_cast<double*>(ys + R * kLdY);
+    float* const grads = parts + (size_t)((int)blockIdx.x % n_parts) * kParams;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gr = lane >> 2, tc = lane & 3;
     // ldmatrix rows and columns of this lane.  A operand with k contiguous, or its transpose from
     // rows of k; B operand with k contiguous (16 columns), or from rows of k
@@ -417,6 +419,19 @@ __global__ void __launch_bounds__(kPassThreads, 1)
     }
 }
 
+// Gradient of parameter i from the partial ones.
+__device__ __forceinline__ float folded(const float* __restrict__ parts, int n_parts, int i) {
+    double sum = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < n_parts; ++k) sum += parts[(size_t)k * kParams + i];
+    return (float)sum;
+}
+
+__global__ void k_fold(const float* __restrict__ parts, int n_parts, float* __restrict__ grads) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kParams) grads[i] = folded(parts, n_parts, i);
+}
+
 // ---------------------------------------------------------------------------------
 // FP32 mode of the training passes, for gradient checks at FP32 accuracy: the same
 // layers and fused epilogues with FP32 operands and activations on the FP32 pipe (no
@@ -554,15 +569,15 @@ __global__ void k_colsum32(int B, int N, const float* __restrict__ dZ, float* __
     atomicAdd(&db[n], s);
 }
 
-// Adam on the FP32 master parameters; the learning rate and the two bias corrections
-// of the iteration are sched[3 * *iter + 0..2].
-__global__ void k_adam(int P, float* __restrict__ p, const float* __restrict__ grad, float* __restrict__ m,
-                       float* __restrict__ v, const float* __restrict__ sched, const unsigned* __restrict__ iter,
-                       float b1, float b2, float eps) {
+// Adam on the FP32 master parameters, from k_pass's partial gradients; the learning rate and the
+// two bias corrections of the iteration are sched[3 * *iter + 0..2].
+__global__ void k_adam(int P, float* __restrict__ p, const float* __restrict__ parts, int n_parts,
+                       float* __restrict__ m, float* __restrict__ v, const float* __restrict__ sched,
+                       const unsigned* __restrict__ iter, float b1, float b2, float eps) {
     const float* sc = sched + 3 * (size_t)*iter;
     const float lr = sc[0], c1 = sc[1], c2 = sc[2];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P; i += gridDim.x * blockDim.x) {
-        const float g = grad[i];
+        const float g = folded(parts, n_parts, i);
         const float mi = b1 * m[i] + (1.f - b1) * g;
         const float vi = b2 * v[i] + (1.f - b2) * g * g;
         m[i] = mi;
@@ -843,6 +858,8 @@ struct mcrt_surrogate {
     size_t in_cap = 0;
     float* d_t = nullptr;  // targets
     size_t t_cap = 0;
+    float* d_parts = nullptr;  // partial gradients
+    size_t parts_cap = 0;
     unsigned seed = 0;
     long long step = 0;
     unsigned char* d_image = nullptr;  // inference image of the current parameters
@@ -877,23 +894,46 @@ LabelTables tables_of(const mcrt_surrogate* s) {
     return LabelTables{s->d_bins, s->d_kext, s->n_bins, s->n_theta, s->n_ktheta};
 }
 
-// Loss and gradients of the B rows in d_in and d_t: gradients of all parameters into d_grads
-// (FP32), the loss added to loss[*iter] (loss[0] without an iteration counter).  Tiles of 16
-// rows while there is an SM for each (a training step of 1024 rows 45 us, 47 with 32), else of
-// 32, which add the weight gradients half as often (2^16 rows: 0.31 ms, 0.45 with 16).
+// How a batch of B rows runs.  Tiles of 16 rows while there is an SM for each (a training step of
+// 1024 rows 45 us, 47 with 32), else of 32, which add the weight gradients half as often (2^16
+// rows: 0.31 ms, 0.45 with 16).  Partial gradients: as many as keep the FP32 sum over the tiles as
+// close to the rows' exact sum as split products did that took in 64 tiles of 128 rows and more.
+// Error of the sum in norm, split products, one sum and these: 512 rows 2.9e-8, 2.6e-8, 1.3e-8; 2048
+// 4.2e-8, 5.5e-8, 1.8e-8; 8192 6.2e-8, 1.6e-7, 3.8e-8; 2^16 2.8e-7, 9.3e-7, 3.8e-8.  More (32) cost 7 us
+// at 8193 rows; up to 8 tiles one is enough, and the call saves 10 us of k_fold.
+struct PassShape {
+    int rows, grid, n_parts;
+    float* parts;
+};
+PassShape pass_shape(const mcrt_surrogate* s, int B) {
+    const int rows = B <= 16 * s->n_sm ? 16 : 32, tiles = (B + rows - 1) / rows;
+    const int n_parts = tiles <= 8 ? 1 : (tiles <= 256 ? 4 : 16);
+    return PassShape{rows, tiles < s->n_sm ? tiles : s->n_sm, n_parts, n_parts == 1 ? s->d_grads : s->d_parts};
+}
+
+// Room for the inputs, the targets and the partial gradients of B rows.
+mcrt_status pass_buffers(mcrt_surrogate* s, int B) {
+    mcrt_status st = ensure(s->d_in, s->in_cap, (size_t)B * kIn * sizeof(float));
+    if (st == MCRT_OK) st = ensure(s->d_t, s->t_cap, (size_t)B * kOut * sizeof(float));
+    const int n_parts = pass_shape(s, B).n_parts;
+    if (st == MCRT_OK && n_parts > 1) st = ensure(s->d_parts, s->parts_cap, sizeof(float) * kParams * n_parts);
+    return st;
+}
+
+// Loss and gradients of the B rows in d_in and d_t: gradients of all parameters into the partial
+// ones (d_grads itself if there is but one), the loss added to loss[*iter] (loss[0] without an iteration counter).
 mcrt_status pass(mcrt_surrogate* s, int B, const LossWeights& w, double* loss, const unsigned* iter) {
-    SK(cudaMemsetAsync(s->d_grads, 0, sizeof(float) * kParams, s->stream));
-    const int small = B <= 16 * s->n_sm, rows = small ? 16 : 32;
-    const int tiles = (B + rows - 1) / rows, grid = tiles < s->n_sm ? tiles : s->n_sm;
+    const PassShape h = pass_shape(s, B);
+    SK(cudaMemsetAsync(h.parts, 0, sizeof(float) * kParams * h.n_parts, s->stream));
     (void)cudaGetLastError();
-    if (small) {
+    if (h.rows == 16) {
         SK(cudaFuncSetAttribute(k_pass<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pass_smem(1)));
-        k_pass<1><<<grid, kPassThreads, pass_smem(1), s->stream>>>(B, s->d_in, s->d_t, w, s->d_wbf, s->d_params,
-                                                                   s->d_grads, loss, iter);
+        k_pass<1><<<h.grid, kPassThreads, pass_smem(1), s->stream>>>(B, s->d_in, s->d_t, w, s->d_wbf, s->d_params,
+                                                                     h.parts, h.n_parts, loss, iter);
     } else {
         SK(cudaFuncSetAttribute(k_pass<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pass_smem(2)));
-        k_pass<2><<<grid, kPassThreads, pass_smem(2), s->stream>>>(B, s->d_in, s->d_t, w, s->d_wbf, s->d_params,
-                                                                   s->d_grads, loss, iter);
+        k_pass<2><<<h.grid, kPassThreads, pass_smem(2), s->stream>>>(B, s->d_in, s->d_t, w, s->d_wbf, s->d_params,
+                                                                     h.parts, h.n_parts, loss, iter);
     }
     SK(cudaGetLastError());
     return MCRT_OK;
@@ -1044,8 +1084,7 @@ mcrt_status mcrt_surrogate_train(mcrt_surrogate* s, int64_t n_steps, int32_t bat
     if (!s || n_steps < 0 || batch < 64 || batch > (1 << 20) || n_steps > (1ll << 31))
         return mcrt_fail_noctx(MCRT_E_INVAL, "mcrt_surrogate_train: bad arguments");
     {
-        mcrt_status st = ensure(s->d_in, s->in_cap, (size_t)batch * kIn * sizeof(float));
-        if (st == MCRT_OK) st = ensure(s->d_t, s->t_cap, (size_t)batch * kOut * sizeof(float));
+        const mcrt_status st = pass_buffers(s, batch);
         if (st != MCRT_OK) return st;
     }
     s->map_valid = false;
@@ -1101,8 +1140,9 @@ mcrt_status mcrt_surrogate_train(mcrt_surrogate* s, int64_t n_steps, int32_t bat
         st = pass(s, batch, w, d_hist, d_iter);
     }
     if (st == MCRT_OK) {
-        k_adam<<<128, 256, 0, s->stream>>>(kParams, s->d_params, s->d_grads, s->d_m, s->d_v, d_sched, d_iter, b1, b2,
-                                           eps);
+        const PassShape h = pass_shape(s, batch);
+        k_adam<<<128, 256, 0, s->stream>>>(kParams, s->d_params, h.parts, h.n_parts, s->d_m, s->d_v, d_sched, d_iter, b1,
+                                           b2, eps);
         k_pack_weights<<<64, 256, 0, s->stream>>>(s->d_params, s->d_wbf, d_iter);
         if (cudaGetLastError() != cudaSuccess) st = MCRT_E_CUDA;
     }
@@ -1218,9 +1258,8 @@ mcrt_status mcrt_surrogate_grad(mcrt_surrogate* s, int64_t n, const float* input
                                 const float* loss_weights, float* grads, double* loss) {
     if (!s || n < 1 || n > (1 << 20) || !inputs || !targets || !grads)
         return mcrt_fail_noctx(MCRT_E_INVAL, "mcrt_surrogate_grad: bad arguments");
-    mcrt_status st = stage_inputs(s, inputs, n);
-    if (st != MCRT_OK) return st;
-    st = ensure(s->d_t, s->t_cap, (size_t)n * kOut * sizeof(float));
+    mcrt_status st = pass_buffers(s, (int)n);
+    if (st == MCRT_OK) st = stage_inputs(s, inputs, n);
     if (st != MCRT_OK) return st;
     SK(cudaMemcpyAsync(s->d_t, targets, (size_t)n * kOut * sizeof(float), cudaMemcpyDefault, s->stream));
     LossWeights w;
@@ -1228,6 +1267,9 @@ mcrt_status mcrt_surrogate_grad(mcrt_surrogate* s, int64_t n, const float* input
     SK(cudaMemsetAsync(s->d_loss, 0, sizeof(double), s->stream));
     st = pass(s, (int)n, w, s->d_loss, nullptr);
     if (st != MCRT_OK) return st;
+    const PassShape h = pass_shape(s, (int)n);
+    if (h.n_parts > 1) k_fold<<<(kParams + 127) / 128, 128, 0, s->stream>>>(h.parts, h.n_parts, s->d_grads);
+    SK(cudaGetLastError());
     SK(cudaMemcpyAsync(grads, s->d_grads, sizeof(float) * kParams, cudaMemcpyDefault, s->stream));
     double l = 0.0;
     SK(cudaMemcpyAsync(&l, s->d_loss, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
@@ -1374,6 +1416,7 @@ mcrt_status mcrt_surrogate_destroy(mcrt_surrogate* s) {
     if (!s) return MCRT_OK;
     if (s->stream) cudaStreamSynchronize(s->stream);
     cudaFree(s->d_t);
+    cudaFree(s->d_parts);
     cudaFree(s->d_bins);
     cudaFree(s->d_kext);
     cudaFree(s->d_params);
