@@ -22,19 +22,21 @@ template <typename T> struct RayCell {
 };
 
 // Cell c of a ray of camera P.cam over the length ell: false when the cell leaves the ray as
-// it is.  The cell's record, grain frame and source are loaded together.
-template <typename T>
+// it is.  The cell's record and grain frame are loaded together, and its source with them
+// (ahead) or once the record says that the cell scatters.
+template <bool ahead, typename T>
 __device__ __forceinline__ bool ray_cell(const ImageParams& P, const V3<T>& Om, const V3<T>& phc, long long c, T ell,
                                          T inv_vol, RayCell<T>& o) {
     const float4 r = __ldg(&P.g.cells[2 * c + 1]);
     float4 q = make_float4(1.f, 0.f, 0.f, 0.f);
     if (P.t.model == MCRT_SCAT_DIPOLE || !P.t.k_iso) q = __ldg(&P.g.cells[2 * c]);
     double2 sa = make_double2(0.0, 0.0), sb = sa;
-    if (P.S) {
+    auto source = [&]() {
         const double2* Sc = reinterpret_cast<const double2*>(P.S + ((size_t)c * P.n_cam + P.cam_index) * 4);
         sa = __ldg(Sc);
         sb = __ldg(Sc + 1);
-    }
+    };
+    if (ahead && P.S) source();
     const T ks = T(r.y);
     const T kext = T(r.x) + ks;
     if (!(kext > T(0) && ell > T(0))) return false;
@@ -62,6 +64,7 @@ __device__ __forceinline__ bool ray_cell(const ImageParams& P, const V3<T>& Om, 
     // emission: the absorption part of K acting on (B, 0, 0, 0)
     T S[4] = {(a1 - s11) * B, (a2 - s12) * B, T(0), T(0)};
     if (P.S && ks > T(0)) {
+        if (!ahead) source();
         const T f = omega * inv_vol;
         T s1 = f * T(sa.y), s2v = f * T(sb.x);
         rotate_qu(s1, s2v, c2, s2);
@@ -80,8 +83,11 @@ __device__ __forceinline__ bool ray_cell(const ImageParams& P, const V3<T>& Om, 
 // lengths) and the four-term step X <- e^{-K dtau} X + W are: the coefficients of a cell, some 400
 // instructions and the loads before them, do not depend on X.  All G lanes walk the next
 // G cells, lane j works out cell j, and the Stokes vector then passes through the cells in
-// order, so the result is that of one lane alone, bit for bit (R: grids with patches).
-template <typename T, int G, bool R>
+// order, so the result is that of one lane alone, bit for bit (R: grids with patches).  One lane
+// takes a cell at a time: as the case G = 1 of the loop for several it held the cell's face beside
+// its coefficients, 60 registers instead of 56 (FP32), and 1024^2 pixels took 2 to 11 % longer
+// than a plain loop.
+template <typename T, int G, bool R, bool ahead>
 __global__ void __launch_bounds__(128) k_image(const __grid_constant__ ImageParams P) {
     constexpr unsigned kAll = 0xffffffffu;
     const int nx = P.npix[0], ny = P.npix[1];
@@ -154,52 +160,69 @@ __global__ void __launch_bounds__(128) k_image(const __grid_constant__ ImagePara
         if (on) descend();
     long long left = (long long)(g.n[0] + g.n[1] + g.n[2]) * (R ? 3 * 16 + 1 : 1) + 3;  // bound on the cells
     T X[4] = {T(0), T(0), T(0), T(0)};
-    while (__any_sync(kAll, on)) {
-        T my_ell = T(0), my_vol = inv_vol_root;
-        long long my_c = -1;
-#pragma unroll 1
-        for (int j = 0; j < G; ++j) {
-            if (!on) continue;
+    auto cell_index = [&]() {
+        return !R || lvl == 0 ? ((long long)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0]
+                              : patch_cell(P.g.patches[lvl - 1], idx[0], idx[1], idx[2]);
+    };
+    // out of the cell, through the face that is ell away along the given axis
+    auto leave_cell = [&](T ell, int axis) {
+        if (!R || lvl == 0) {
+            on = cross_face(g, idx, p, dir, ell, axis);
+            if constexpr (R)
+                if (on) descend();
+        } else if (!cross_face(gc, idx, p, dir, ell, axis)) {
+            // out of the patch: the root cell beyond its face
+            const PatchDev& pq = P.g.patches[lvl - 1];
+            for (int a = 0; a < 3; ++a) idx[a] = pq.box[a] + (a == axis ? 0 : idx[a] / pq.factor);
+            idx[axis] = dir[axis] > T(0) ? pq.box[3 + axis] : pq.box[axis] - 1;
+            lvl = 0;
+            gc = g;
+            inv_vol = inv_vol_root;
+            on = idx[axis] >= 0 && idx[axis] < g.n[axis];
+            if (on) descend();
+        }
+    };
+    auto through = [&](const RayCell<T>& rc) {
+        rotate_qu(X[1], X[2], rc.c2, rc.s2);
+        cell_step(rc.k, X);
+        rotate_back(X[1], X[2], rc.c2, rc.s2);
+    };
+    if constexpr (G == 1) {
+        while (on) {
             int axis;
             const T ell = exit_distance(gc, idx, p, dir, axis);
-            if (axis < 0 || left-- <= 0) {
-                on = false;
-                continue;
-            }
-            if (j == j_me) {
-                my_ell = ell;
-                my_vol = inv_vol;
-                my_c = !R || lvl == 0 ? ((long long)idx[2] * g.n[1] + idx[1]) * g.n[0] + idx[0]
-                                      : patch_cell(P.g.patches[lvl - 1], idx[0], idx[1], idx[2]);
-            }
-            if (!R || lvl == 0) {
-                on = cross_face(g, idx, p, dir, ell, axis);
-                if constexpr (R)
-                    if (on) descend();
-            } else if (!cross_face(gc, idx, p, dir, ell, axis)) {
-                // out of the patch: the root cell beyond its face
-                const PatchDev& pq = P.g.patches[lvl - 1];
-                for (int a = 0; a < 3; ++a) idx[a] = pq.box[a] + (a == axis ? 0 : idx[a] / pq.factor);
-                idx[axis] = dir[axis] > T(0) ? pq.box[3 + axis] : pq.box[axis] - 1;
-                lvl = 0;
-                gc = g;
-                inv_vol = inv_vol_root;
-                on = idx[axis] >= 0 && idx[axis] < g.n[axis];
-                if (on) descend();
-            }
+            if (axis < 0 || left-- <= 0) break;
+            RayCell<T> rc;
+            if (ray_cell<ahead>(P, Om, phc, cell_index(), ell, inv_vol, rc)) through(rc);
+            leave_cell(ell, axis);
         }
-        RayCell<T> rc;
-        const bool act = my_c >= 0 && ray_cell(P, Om, phc, my_c, my_ell, my_vol, rc);
-        const unsigned any = __ballot_sync(kAll, act);
+    } else {
+        while (__any_sync(kAll, on)) {
+            T my_ell = T(0), my_vol = inv_vol_root;
+            long long my_c = -1;
 #pragma unroll 1
-        for (int j = 0; j < G; ++j) {
-            if (act && j == j_me) {
-                rotate_qu(X[1], X[2], rc.c2, rc.s2);
-                cell_step(rc.k, X);
-                rotate_back(X[1], X[2], rc.c2, rc.s2);
+            for (int j = 0; j < G; ++j) {
+                if (!on) continue;
+                int axis;
+                const T ell = exit_distance(gc, idx, p, dir, axis);
+                if (axis < 0 || left-- <= 0) {
+                    on = false;
+                    continue;
+                }
+                if (j == j_me) {
+                    my_ell = ell;
+                    my_vol = inv_vol;
+                    my_c = cell_index();
+                }
+                leave_cell(ell, axis);
             }
-            if constexpr (G > 1) {
-                static_assert(G == 4 || G == 8);
+            RayCell<T> rc;
+            const bool act = my_c >= 0 && ray_cell<ahead>(P, Om, phc, my_c, my_ell, my_vol, rc);
+            const unsigned any = __ballot_sync(kAll, act);
+#pragma unroll 1
+            for (int j = 0; j < G; ++j) {
+                if (act && j == j_me) through(rc);
+                static_assert(G == 1 || G == 4 || G == 8);
                 constexpr unsigned kGroups = G == 8 ? 0x01010101u : 0x11111111u;  // lane 0 of each ray
                 if (any & (kGroups << j)) {
 #pragma unroll
@@ -622,31 +645,39 @@ cudaError_t launch_dipole_setup(double eps_re, double eps_im, double aspect, dou
     return cudaGetLastError();
 }
 
-template <typename T, int G> static void image_launch(const ImageParams& p, int block, cudaStream_t s) {
+template <typename T, int G, bool ahead = true> static void image_launch(const ImageParams& p, int block, cudaStream_t s) {
     const long long threads = (long long)p.npix[0] * p.npix[1] * G;
     const unsigned grid = (unsigned)((threads + block - 1) / block);
     if (p.g.n_patches > 0)
-        k_image<T, G, true><<<grid, block, 0, s>>>(p);
+        k_image<T, G, true, ahead><<<grid, block, 0, s>>>(p);
     else
-        k_image<T, G, false><<<grid, block, 0, s>>>(p);
+        k_image<T, G, false, ahead><<<grid, block, 0, s>>>(p);
 }
 
 // Lanes per ray: the fewer rays, the more of a ray's cells are worked out at once; with enough
 // rays to fill the SMs the shared walk only repeats work.  Measured per image, us with 8, 4 and 1
-// lanes (and one ray per lane before): FP32, 96^3 disk, 64^2 81, 101, 256 (271); 128^2 125, 122,
-// 245 (301); 181^2 204, 150, 238 (286); 256^2 361, 246, 247 (293); FP64, 24^3 disk, 32^2 96, 135,
-// 325 (326); 64^2 174, 131, 326 (327); 128^2 590, 408, 319 (320).  Blocks of 64 keep FP64's last
-// wave short (256^2: 801 us against 856 with 128); pixel tiles of 8 x 4 per warp gave FP32 no more
-// than 2 % at 512^2 and lost 6 % at 256^2 against rows.
+// lanes (and the one-lane loop that read a cell's record first): FP32, 96^3 disk, 64^2 81, 101, 256
+// (271); 128^2 125, 122, 245 (301); 181^2 204, 150, 238 (286); 256^2 361, 246, 228 (293); FP64, 24^3
+// disk, 32^2 96, 135, 325 (326); 64^2 174, 131, 326 (327); 128^2 590, 408, 319 (320).
+// One lane per ray in blocks of 128: of 64, FP64 images of 256^2 pixels took 0.94 to 1.38 of the
+// time (64^3 disk and slab), 512^2 as much.  Pixel tiles of 8 x 4 per warp gave FP32 no more than
+// 2 % at 512^2 and lost 6 % at 256^2 against rows.
+// A cell's source with its record, or after it: together the latency is paid once (FP32, 64^3
+// disk, 256^2 228 us against 248; plane-parallel slab 188 against 216); from some 10^5 rays on bytes
+// count, and cells that do not scatter need none (1024^2: disk 1280 against 1276, sphere 1097 against
+// 1080, refined disk 1459 against 1427, absorbing slab 609 against 560).
 template <typename T> static void image_launch(const ImageParams& p, cudaStream_t s) {
     constexpr long long kRays8 = sizeof(T) == 4 ? 12288 : 2048, kRays4 = sizeof(T) == 4 ? 40960 : 8192;
+    constexpr long long kRaysAhead = 1ll << 17;
     const long long rays = (long long)p.npix[0] * p.npix[1];
     if (rays <= kRays8)
         image_launch<T, 8>(p, 64, s);
     else if (rays <= kRays4)
         image_launch<T, 4>(p, 128, s);
+    else if (sizeof(T) == 8 || rays <= kRaysAhead)
+        image_launch<T, 1>(p, 128, s);
     else
-        image_launch<T, 1>(p, sizeof(T) == 4 ? 128 : 64, s);
+        image_launch<float, 1, false>(p, 128, s);
 }
 
 cudaError_t launch_image(const ImageParams& p, int precision, cudaStream_t s) {
