@@ -103,9 +103,10 @@ bool is_device_ptr(const void* p) {
 }
 
 // Device copies of a caller's buffers: a buffer itself if it is device memory, else its
-// part of one temporary allocation, filled from host memory.  An allocation and its free
-// cost 60 us and more whatever their size, as much as a small model's set-up kernels, so
-// what lives together is allocated together here and below.
+// part of one temporary allocation, filled from host memory.  An allocation that takes
+// pages of its own costs 60 us and more with its free, as much as a small model's set-up
+// kernels, so what lives together is allocated together here and below, unless that takes a
+// page more.
 struct DevIn {
     void* owned = nullptr;
     ~DevIn() {

@@ -176,9 +176,9 @@ template <typename T> struct Pair {
     T a, b;
 };
 // (A, B) over the larger of them, (1, 0) for zeros: a function of its own, since the two divisions
-// hardly ever run and stood in every rotation (plane-parallel slab 365 -> 352 ms, 64^3 disk's
-// transport 3.83 -> 3.63 and tally 2.37 -> 2.20 ms, batched sweep 163.7 -> 155 ms, together with
-// the rotations that cannot need it)
+// hardly ever run and stood in every rotation (4 % off the plane-parallel slab, 5 % off the
+// transport and 7 % off the tally of the 64^3 disk, together with the rotations that cannot need it;
+// inlined in FP64, the 24^3 disk takes 5 % longer)
 template <typename T> __device__ __noinline__ Pair<T> rescaled(T A, T B) {
     const T m = fmax(fabs(A), fabs(B));
     if (!(m > T(0))) return Pair<T>{T(1), T(0)};
@@ -251,15 +251,15 @@ template <typename T> __device__ __forceinline__ T e1(T x) {
 
 // The sine and cosine that only media with a circular-retardance element (a3 != 0) need: a function
 // of its own, so that its slow path, with the stack that takes, stays out of the walk of everything
-// else (refined disk's transport 82.1 -> 78.9 ms, plane-parallel slab 383 -> 376 ms).
+// else (4 % off the refined disk's transport, 2 % off the plane-parallel slab).
 template <typename T> __device__ __noinline__ Pair<T> sincos_apart(T y) {
     Pair<T> p;
     t_sincos(y, &p.a, &p.b);
     return p;
 }
 
-// With `calls` false inlined, for the surrogate's transport, where every segment needs it (64^3 disk,
-// 42 rounds: 7.50 -> 7.32 ms).
+// With `calls` false inlined, for the surrogate's transport, where every segment needs it (2 % off
+// the 64^3 disk's).
 template <bool calls, typename T> __device__ __forceinline__ Pair<T> sincos_of(T y) {
     if constexpr (calls) return sincos_apart(y);
     Pair<T> p;
@@ -281,10 +281,9 @@ template <bool calls, typename T> __device__ __forceinline__ Pair<T> e1_turning(
     return Pair<T>{t_mul(mad2(nr, x, ni, y), den), t_mul(msb2(nr, y, ni, x), den)};
 }
 // The same as a function of its own, for the in-place kernels: few media turn U and V, and without
-// this code in their loop the batched sweep takes 150.8 instead of 154.8 ms and the plane-parallel
-// slab 347.7 instead of 352.2 (a slab that does turn them, 1e6 packets, 20.2 instead of 19.9).  The
-// table rounds are faster with it inlined (refined disk's transport 78.6 against 79.8 ms), as are
-// the surrogate's, whose media all turn (7.6 against 7.8 ms).
+// this code in their loop the batched sweep takes 2.6 % less and the plane-parallel slab 1.3 % (a slab
+// that does turn them 1.5 % more).  The table rounds are faster with it inlined (refined disk's
+// transport by 1.5 %), as are the surrogate's, whose media all turn (2.5 %).
 template <typename T> __device__ __noinline__ Pair<T> e1_turning_apart(T x, T y) { return e1_turning<true>(x, y); }
 
 template <bool apart, bool calls, typename T> __device__ __forceinline__ void e1_complex(T x, T y, T& re, T& im) {

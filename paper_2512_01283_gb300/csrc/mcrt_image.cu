@@ -656,11 +656,11 @@ template <typename T, int G, bool ahead = true> static void image_launch(const I
 
 // Lanes per ray: the fewer rays, the more of a ray's cells are worked out at once; with enough
 // rays to fill the SMs the shared walk only repeats work.  Measured per image, us with 8, 4 and 1
-// lanes (and the one-lane loop that read a cell's record first): FP32, 96^3 disk, 64^2 81, 101, 256
-// (271); 128^2 125, 122, 245 (301); 181^2 204, 150, 238 (286); 256^2 361, 246, 228 (293); FP64, 24^3
-// disk, 32^2 96, 135, 325 (326); 64^2 174, 131, 326 (327); 128^2 590, 408, 319 (320).
-// One lane per ray in blocks of 128: of 64, FP64 images of 256^2 pixels took 0.94 to 1.38 of the
-// time (64^3 disk and slab), 512^2 as much.  Pixel tiles of 8 x 4 per warp gave FP32 no more than
+// lanes (and one that read source and frame after the record): FP32, 96^3 disk, 64^2 66, 75, 164
+// (206); 128^2 110, 101, 180 (195); 181^2 187, 134, 170 (194); 256^2 330, 230, 191 (217); FP64, 24^3
+// disk, 32^2 92, 125, 292 (298); 64^2 158, 124, 292 (298); 128^2 543, 374, 290 (299).
+// One lane per ray in blocks of 128: of 64, FP64 images of 256^2 pixels took 0.94 (64^3 disk) to
+// 1.38 (slab) of the time, those of 512^2 0.99.  Pixel tiles of 8 x 4 per warp gave FP32 no more than
 // 2 % at 512^2 and lost 6 % at 256^2 against rows.
 // A cell's source with its record, or after it: together the latency is paid once (FP32, 64^3
 // disk, 256^2 228 us against 248; plane-parallel slab 188 against 216); from some 10^5 rays on bytes

@@ -69,12 +69,11 @@ __device__ __forceinline__ void red_add(double* p, double v) {
 // rows and places, which other lanes staged, before their reads here, and these reads before
 // the next rows; neither a ballot nor a warp reduction does.
 //
-// The in-place kernels issue instructions, not bytes (65 to 69 % of the issue slots, 0.03 % of
+// The in-place kernels issue instructions, not bytes (58 to 71 % of the issue slots, 0.05 % of
 // DRAM on the plane-parallel slab).  A bulk reduction per lane has uniform operands, so the
 // warp issued it for one lane after the other; here a warp's rows of 1 or 2 cameras take 4
-// or 8 coalesced reductions.  Measured on 1e7 packets: plane-parallel slab 513 -> 481 ms,
-// spheroids 75.2 -> 70.4 ms, the sweep's 32 jobs of 5e5 packets 221 -> 193 ms (one camera); with
-// 8 cameras 8.75 -> 8.47 ms (3e5-packet slab).  The table rounds' tally kernel, 8 cameras and
+// or 8 coalesced reductions.  When introduced it took 6 % off the plane-parallel slab and the
+// spheroids (2 cameras), 13 % off the batched sweep (1 camera) and 3 % off a slab with 8.  The table rounds' tally kernel, 8 cameras and
 // rows beyond L2, keeps its bulk reductions (585 ms against 615 per 1e8-packet disk step:
 // 1.08e10 rows/s against 1.03e10 at spread positions).
 template <typename T, typename At>

@@ -30,8 +30,10 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kDefaultBlock = 128;
-// resident blocks per SM the FP32 kernels are compiled for (register budget 96);
-// shared memory (tables + 272 B of tally staging per thread) allows 5 such blocks
+// resident blocks per SM the FP32 in-place kernels are compiled for (5: 96 registers).  With 4,
+// 5 and 6, ms: plane-parallel slab of 1e7 packets 370, 339, 330; spheroids 73.1, 65.3, 68.2; batched
+// sweep 167, 151, 160.  Shared memory (tables and 32 rows of 16 B per camera and warp) allows 5 up
+// to 16 cameras with tables of 181 angles.
 #ifndef MCRT_MIN_BLOCKS
 #define MCRT_MIN_BLOCKS 5
 #endif
@@ -41,15 +43,18 @@ constexpr int kDefaultBlock = 128;
 // only delayed the last ones).  The more often packets scatter the sooner a larger group is
 // together; what waiting lanes idle meets the phase's cost at these counts, measured on GB300
 // with the trials spread over the warp:
-//   Rayleigh 8: plane-parallel slab (41 scatterings a packet) 405 ms, 431 with 4 and 406 with 10;
-//   spheroids and FP64 tables 4: spheroid sphere (0.6 scatterings a packet) 69.3 ms, 70.0 with 3,
-//     72.3 with 8; FP64 disk of 1e5 packets 12.2 ms, 13.3 with 8;
-//   table rounds 6: transport of 5e6 star and 5e6 thermal packets of the 192^3 disk 42.4 + 24.8 ms,
-//     42.8 + 24.9 with 5 and 42.7 + 24.8 with 8;
-//   batched launches 8 (9.4e9 events/s on the 256-job sweep, 8.7e9 with 4).
-// New packets are taken by 4 lanes together (5: slab 409 ms; singly: batched sweep 7.5e9 events/s
-// against 8.7e9); a rule on the lane steps spent waiting, instead of the counts, came within 3 %
-// on every workload but was better on none.
+//   Rayleigh 8: plane-parallel slab (41 scatterings a packet) 339 ms, 349 with 4 and 340 with 10; a
+//     sphere of optical depth 5 11.1 ms, 11.5 with 4.  Media that scatter little would take 4:
+//     spheres of depth 1 3.98 ms (3.94) and 0.1 2.79 ms (2.65); the launch does not know the depth;
+//   spheroids and FP64 tables 4: spheroid sphere (0.6 scatterings a packet) 65.3 ms, 64.8 with 3 and
+//     68.5 with 8, but of depth 5 7.71, 7.96 and 7.55; FP64 disk of 1e5 packets 9.9 with each;
+//   table rounds 6: transport of 1e7 packets of the refined disk 74.1 ms, 74.3 with 5 and 74.7 with
+//     8; of the 192^3 disk 59.0 with each;
+//   batched launches 8: sweep 151 ms, 157 with 4.
+// New packets are taken by 4 lanes together, with 2, 4 and 6: slab 337, 339, 345 ms; sweep 156, 151,
+// 151; transport of the 192^3 disk 64.5, 59.0, 57.6 and of the refined one 73.4, 74.1, 75.2.  A rule on
+// the lane steps spent waiting, instead of the counts, came within 3 % on every workload but was
+// better on none.
 #ifndef MCRT_SCATTER_BATCH
 #define MCRT_SCATTER_BATCH 4
 #endif
@@ -98,9 +103,8 @@ constexpr unsigned kRecChunk = 32u * MCRT_REC_CHUNK;
 #define MCRT_ABS_GROUPS 0
 #endif
 // In-place kernels: same-cell lanes pre-sum their source and absorbed terms (1) or
-// every lane reduces its own (0).  Without the match: batched sweep 9.6e9 -> 1.1e10
-// events/s, plane-parallel slab 1.15e10 -> 1.25e10, spheroids 1.54e10 -> 1.76e10,
-// refined disk 3.8e9 -> 5.1e9.
+// every lane reduces its own (0).  Without the match, when introduced: batched sweep 15 %
+// more events/s, plane-parallel slab 9 %, spheroids 14 %, refined disk 34 %.
 #ifndef MCRT_INPLACE_GROUPS
 #define MCRT_INPLACE_GROUPS 0
 #endif
@@ -428,8 +432,8 @@ __device__ bool emit(const TransportParams& P, const JobRef<T, B>& job, long lon
 }
 
 // emit() as a function of its own, returning the packet: inlined, the births of all source kinds
-// stood in the middle of the in-place kernels' loop (plane-parallel slab 375 -> 363 ms, batched
-// sweep 162.5 -> 159.6 ms; slab of 1e6 packets 1.14 -> 1.16 ms).
+// stood in the middle of the in-place kernels' loop (plane-parallel slab 3 % less, batched sweep 2 %;
+// the absorbing slab, where births count, 2 % more).
 template <typename T, bool B, bool WP> struct Born {
     Packet<T> pk;
     bool inside;
@@ -542,9 +546,8 @@ __device__ __noinline__ void tally_apart(const TransportParams& P, const T* cams
 // ends here leaves its fate (finish()'s flag) to the kernel's loop, which holds the only copy of
 // that code.  The instruction cache is what such code costs
 // (22 % of the stalls of the table rounds were instruction fetches): one copy instead of four,
-// with the parts of mcrt_device.cuh that are called apart, took 12 to 14 kB off the kernels and
-// the refined disk's transport from 85.8 to 78.6 ms, the plane-parallel slab from 402 to 376 ms,
-// the batched sweep from 171.7 to 165 ms.
+// with the parts of mcrt_device.cuh that are called apart, took 12 to 14 kB off the kernels, 8 % off
+// the refined disk's transport, 6 % off the plane-parallel slab and 4 % off the batched sweep.
 template <typename T, int SCAT, bool B, bool R, bool ISO>
 __device__ __forceinline__ void step(const TransportParams& P, const Smem<T>& sm, Packet<T>& pk, bool& alive,
                                      int& fate, unsigned work, int& staged) {
@@ -935,8 +938,7 @@ __device__ __forceinline__ bool table_trial(const TablesDev& tabs, int bin, cons
     }
     const int j = lo;
     // the interval's limits from the table: two sine-cosine calls and two divisions fewer per
-    // trial (table-round transport 99.1 -> 94.3 ms on the refined disk's 1e7 packets, FP64 disk
-    // of 1e5 packets 13.3 -> 12.6 ms)
+    // trial (5 % of the refined disk's transport and of the FP64 disk of 1e5 packets)
     const T c0 = entry_at<T>(tabs.cos_d, tabs.cos_f, j), c1 = entry_at<T>(tabs.cos_d, tabs.cos_f, j + 1);
     mu = c0 - ut.b * (c0 - c1);
     T sn = (T(1) - mu) * (T(1) + mu);
@@ -952,8 +954,8 @@ __device__ __forceinline__ bool table_trial(const TablesDev& tabs, int bin, cons
 }
 
 // One trial of the rejection sampling of a dipole (Rayleigh) scattering: isotropic proposal
-// in the grain frame (3 / 4 of the trials' constant is the peak of P11), accepted like a
-// tabulated one.
+// in the grain frame, accepted like a tabulated one.  The trials' constant is twice P11's peak,
+// 3 / (8 pi), which covers I + |Q|.
 template <typename T>
 __device__ __forceinline__ bool rayleigh_trial(const float4& q, const Draw4<T>& ut, const V3<T>& n, const V3<T>& th,
                                                const V3<T>& ph, const T X[4], V3<T>& n2) {
@@ -1010,8 +1012,8 @@ template <typename T> __device__ __forceinline__ V3<T> shfl3(const V3<T>& v, int
 // order, and the packet takes its first accepted trial.  Direction, matrix and trial count are
 // thus those of the sequential rule (same random numbers, same arithmetic; V is passed
 // where a trial reads it, for aligned spheroids).  All 32 lanes call it.  Measured against
-// every lane looping over its own trials: plane-parallel slab, 1e7 packets, 480 -> 431 ms
-// (groups of 4), spheroids 70.2 -> 69.5 ms.
+// every lane looping over its own trials: 10 % off the plane-parallel slab (groups of 4), 1 % off
+// the spheroids.
 template <typename T, int SCAT, bool B>
 __device__ __forceinline__ void scatter_coop(const TransportParams& P, const Smem<T>& sm, Packet<T>& pk, bool& alive,
                                              int& fate) {
@@ -1162,8 +1164,8 @@ __device__ __forceinline__ int job_index(const TransportParams& P, long long gpi
 }
 
 // resident blocks per SM of the table-round instantiation: without the camera loop
-// and its staging slots it fits more warps per SM.  6 (80 registers, almost no spills) against 7
-// and 8, ms: 1e7 star packets of the 192^3 disk 38.5, 39.4, 41; refined disk 73.7, 74.3, 89
+// and its staging slots it fits more warps per SM.  With 5, 6 (80 registers, almost no spills) and
+// 7, ms: 1e7 packets of the 192^3 disk 59.5, 59.0, 60.2; of the refined disk 77.0, 74.1, 74.8
 #ifndef MCRT_ROUND_MIN_BLOCKS
 #define MCRT_ROUND_MIN_BLOCKS 6
 #endif
@@ -1174,7 +1176,7 @@ constexpr int min_blocks() {
 
 // ISO: the extinction does not depend on direction or polarization (spherical grains), so that a
 // segment needs one exponential for the three eigenvalues and neither the grain frame nor the
-// extinction table: sphere of 1e5 packets 0.58 -> 0.49 ms; kernels apart, because as a branch
+// extinction table: 15 % off a sphere of 1e5 packets (0.54 ms); kernels apart, because as a branch
 // the extra code cost the others 2 to 6 %.  The jobs of a batched launch may differ in it.
 template <typename T, int SCAT, bool B, bool R, bool ISO>
 __global__ void __launch_bounds__(kDefaultBlock, (min_blocks<T, SCAT>()))

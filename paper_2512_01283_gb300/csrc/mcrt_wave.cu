@@ -904,10 +904,11 @@ __global__ void __launch_bounds__(tc::kRows * kScatGroups, 1) k_sur_scatter_tc(c
 // share nothing, so no lane waits for another.  Same arithmetic as the in-place tally
 // of k_transport (table_matrix, plane_rotation, apply_plane).
 // One staging row per lane: a second one, alternated from tile to tile, lets the reduction of the
-// tile before drain, but halves the warps that fit (8 cameras: 24 warps per SM against 12).  ms
-// with two rows and blocks of 128, with one and 128, with one and 256 and the records streamed
-// past the L2: 64^3 disk 2.20, 2.12, 2.09; refined disk 53.8, 53.1, 52.0; 192^3 disk, 1e7 packets,
-// 60.0, 58.4, 57.6.  Blocks of 64 and fewer of them per SM were slower.
+// tile before drain, but halves the warps that fit (8 cameras: 24 warps per SM against 12).  ms with
+// two rows and blocks of 128 and with one, blocks of 256 and the records streamed past the L2:
+// 64^3 disk 2.60, 2.48; refined disk 53.3, 51.6; 192^3 disk of 1e7 packets, 8 cameras 58.0, 58.0, 4
+// cameras 32.8, 31.9; 128^3 disk, 16 cameras (8 warps per SM against 4) 165, 74.  Blocks of 64 and
+// fewer of them per SM were slower.
 constexpr int kTabBlock = 256;
 // a lane's staging row: the cameras' rows, padded by 16 B so that the 16-byte stores of
 // a quarter-warp's lanes (rows 8 c + 4 words apart) fall in different bank groups
