@@ -1,6 +1,8 @@
 """GPU: a model whose cell records fill whole 2 MiB pages takes no page beyond them.  What is
 kept beside the records is small and shares the page of the other small allocations; in one
 allocation with them it cost a page, and a creation 10 % longer."""
+import gc
+
 import pytest
 
 from paper_2512_01283_gb300 import build as B
@@ -19,6 +21,7 @@ def test_cells_of_whole_pages_take_no_page_more(n):
     model = dict(host, **{k: torch.from_numpy(host[k]).cuda() for k in ("kappa_abs", "kappa_sca", "bfield")
                           if host.get(k) is not None})
     first = M.Model(model)  # loads the set-up kernels and opens the page of the small allocations
+    gc.collect()
     torch.cuda.synchronize()
     before = torch.cuda.mem_get_info()[0]
     second = M.Model(model)
